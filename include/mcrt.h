@@ -474,16 +474,16 @@ MCRT_API int mcrt_tally_read_sums(const mcrt_tally* tally, double* s1, double* s
  * [2] real collisions, [3] ground hits, [4] leaf steps on paths,
  * [5] tentative collisions on sun rays, [6] leaf steps on sun rays,
  * [7] sun rays, [8] aborted paths (step guard), [9] free flights started,
- * and, when n >= 13: [10] most loop iterations spent on one path, [11] the
- * longest time in ns a GPU warp ran before the work queue ran dry, [12] the
- * longest time in ns a warp ran in total, and when n >= 22, [13..21] SM
- * clock cycles summed over warps spent in the sections of the trace loop
- * (loop top, random block, path start, ray start, step, vertex, load,
- * after-load, ray/path end), and when n >= 30, [22..29] lane occupancy
- * summed over warp iterations: iterations, lanes holding a path, lanes
- * taking a traversal step, of those at a tentative collision, lanes running
- * a batched rare phase (path start, ray start, vertex), lanes waiting for
- * one, iterations that ran rare phases, lanes with no path.  n >= 10. */
+ * and, when n >= 13: [10] most step iterations and rare passes spent on one
+ * path, [11] the longest time in ns a GPU warp ran before the work queue ran
+ * dry, [12] the longest time in ns a warp ran in total, and when n >= 22,
+ * [13..21] SM clock cycles summed over warps spent in the sections of the
+ * trace loop (sums and claims, random block, path start, ray start, steps,
+ * vertex, two zeros, ended rays and paths), and when n >= 30, [22..29] lane
+ * occupancy summed over step iterations: iterations, lanes holding a path,
+ * lanes taking a traversal step, of those at a tentative collision, lanes
+ * running in a rare pass (path start, ray start, vertex, ended ray), lanes
+ * waiting for one, rare passes, lanes with no path.  n >= 10. */
 MCRT_API int mcrt_tally_counters(const mcrt_tally* tally, uint64_t* counters, size_t n);
 
 /* Device time of the trace kernel that filled the tally, in ms. */

@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <vector>
 #include <utility>
@@ -58,6 +59,14 @@ void dfree(mcrt_ctx* ctx, void* p)
 
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
+void set_sun(DevScene& S, const float sun[3])
+{
+    for (int a = 0; a < 3; ++a) {
+        S.sun[a] = sun[a];
+        S.inv_sun[a] = sun[a] != 0.0f ? 1.0f / sun[a] : std::numeric_limits<float>::quiet_NaN();
+    }
+}
+
 bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
 
 }  // namespace
@@ -94,7 +103,7 @@ DevScene make_dev_scene(const mcrt_scene* sc, float k_gas)
     S.k_gas = k_gas;
     S.albedo = sc->albedo;
     S.rayleigh = sc->clear_phase == MCRT_PHASE_RAYLEIGH;
-    for (int a = 0; a < 3; ++a) S.sun[a] = sc->sun[a];
+    set_sun(S, sc->sun);
     if (sc->d_hf) {
         S.hf = sc->d_hf;
         S.hpyr = sc->d_hpyr;
@@ -738,7 +747,7 @@ int run_trace(mcrt_scene* sc, TraceParams& P, int sensor, const mcrt_trace_opts*
     const int block = o->block_size ? o->block_size : 128;
     int grid = o->grid_size;
     if (!grid) grid = ctx->sm_count * trace_blocks_per_sm(sensor, bf16, count, P.S.hf != nullptr, P.sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh, block);
-    if (!o->chunk) P.chunk = auto_chunk(P.total, (unsigned long long)grid * block, sensor == kCamera ? P.spp : 0u);
+    if (!o->chunk) P.chunk = auto_chunk(P.total, ctx->sm_count, o->grid_size, block, sensor == kCamera ? P.spp : 0u);
     P.s1 = t->d_s1;
     P.s2 = t->d_s2;
     P.counters = t->d_counters;
@@ -873,7 +882,7 @@ int run_learned(mcrt_scene* sc, const TraceParams& P0, int sensor, const mcrt_tr
             P.total = r == 0 ? nb : n_in;
             P.chunk = r > 0 ? 1u
                             : (o->chunk ? P0.chunk
-                                        : auto_chunk(nb, (unsigned long long)grid * block,
+                                        : auto_chunk(nb, ctx->sm_count, o->grid_size, block,
                                                      sensor == kCamera ? (uint32_t)spp : 0u));
             P.qin = qin; P.qin_feat = fin_feat; P.qin_mix = mix;
             P.qout = qout; P.qout_feat = fout; P.qout_count = cnt; P.qout_cap = (unsigned)nb;
@@ -1182,9 +1191,8 @@ int prepare_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, const 
         if (rc) return rc;
         h[i].S = make_dev_scene(sc, it.k_gas);
         const double z = it.sun_zenith_deg * M_PI / 180.0, a = it.sun_azimuth_deg * M_PI / 180.0;
-        h[i].S.sun[0] = (float)(std::sin(z) * std::cos(a));
-        h[i].S.sun[1] = (float)(std::sin(z) * std::sin(a));
-        h[i].S.sun[2] = (float)std::cos(z);
+        const float sun[3] = {(float)(std::sin(z) * std::cos(a)), (float)(std::sin(z) * std::sin(a)), (float)std::cos(z)};
+        set_sun(h[i].S, sun);
         h[i].begin = begin;
         h[i].npaths = it.npaths;
         h[i].key = make_uint2((uint32_t)it.seed, (uint32_t)(it.seed >> 32));

@@ -149,7 +149,7 @@ struct LevelTable {
 // lb: log2 of the branching per axis (3 pyramid, 1 octree); a level-L cell
 // spans 2^(lb L) voxels per axis, which is the shift the entry records.
 __global__ void __launch_bounds__(256) leafmap_kernel(LevelTable T, int levels, int finest, float tau, int lb,
-                                                      int n1x, int n1y, int n1z, uint2* __restrict__ leaf)
+                                                      int n1x, int n1y, int n1z, int nbx, int nby, uint2* __restrict__ leaf)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)n1x * n1y * n1z) return;
@@ -167,7 +167,10 @@ __global__ void __launch_bounds__(256) leafmap_kernel(LevelTable T, int levels, 
         }
     }
     if (finest == 0) {
-        leaf[i] = make_uint2(0u, 0u);
+        // voxel leaves: the majorant is the voxel itself, so the entry names the cell's brick
+        const int sb = 3 - lb;
+        leaf[i] = make_uint2(((uint32_t)(cz >> sb) * (uint32_t)nby + (uint32_t)(cy >> sb)) * (uint32_t)nbx +
+                             (uint32_t)(cx >> sb), 0u);
     } else {
         const int s = lb * (finest - 1);
         const size_t c = ((size_t)(cz >> s) * T.dims[finest][1] + (cy >> s)) * T.dims[finest][0] + (cx >> s);
@@ -276,7 +279,7 @@ cudaError_t launch_leafmap(const mcrt_scene* sc, float tau, int finest, int grid
     const int* n1 = oct ? &sc->oct_dims[3] : sc->nb;
     const long long cells = (long long)n1[0] * n1[1] * n1[2];
     leafmap_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(T, levels, finest, tau, lb, n1[0], n1[1], n1[2],
-                                                                      oct ? sc->d_oleaf : sc->d_leaf);
+                                                                      sc->nb[0], sc->nb[1], oct ? sc->d_oleaf : sc->d_leaf);
     return cudaGetLastError();
 }
 

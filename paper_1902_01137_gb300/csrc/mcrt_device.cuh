@@ -98,13 +98,14 @@ struct DevScene {
     int nb[3];           // bricks (8^3 voxels) per axis == level-1 cells
     const float* __restrict__ vox;       // brick-major FP32 field, or null
     const uint16_t* __restrict__ vox16;  // brick-major BF16 field, or null
-    const uint2* __restrict__ leaf;      // per level-1 cell: {majorant bits, minorant | leaf shift}
+    const uint2* __restrict__ leaf;      // per level-1 cell: {majorant bits, minorant | leaf shift}; voxel leaves: {brick, 0}
     int lb;              // log2 of the grid's branching per axis: 3 (8^L pyramid) or 1 (2^L octree)
     int nl[3];           // level-1 cells per axis of the tracked grid (leaf-map dims)
     float k_clear, ssa_clear, ssa_cloud, g;
     float k_gas;         // extra uniform pure absorber
     float albedo;        // Lambertian ground
     float sun[3];        // unit vector toward the sun
+    float inv_sun[3];    // its reciprocals as dir_rcp gives them
     int rayleigh;        // clear air scatters with the Rayleigh phase function (else HG with g)
     // heightfield ground (hf null: flat ground at z = 0).  Heights sit at
     // the corners of a periodic grid of hn[0] x hn[1] cells; hpyr holds the
@@ -123,9 +124,10 @@ struct DevScene {
 
 __device__ __forceinline__ size_t brick_index(const DevScene& S, int i, int j, int k)
 {
-    const size_t b = ((size_t)(k >> 3) * (size_t)S.nb[1] + (size_t)(j >> 3)) * (size_t)S.nb[0] + (size_t)(i >> 3);
+    // (brick counts fit 32 bits: a brick is at least 1 KiB)
+    const uint32_t b = ((uint32_t)(k >> 3) * (uint32_t)S.nb[1] + (uint32_t)(j >> 3)) * (uint32_t)S.nb[0] + (uint32_t)(i >> 3);
     const uint32_t off = ((((uint32_t)k & 7u) << 3 | ((uint32_t)j & 7u)) << 3) | ((uint32_t)i & 7u);
-    return b * 512u + off;
+    return (unsigned long long)b * 512u + off;
 }
 
 template <bool BF16>
@@ -148,9 +150,9 @@ __device__ __forceinline__ float kfetch(const DevScene& S, int i, int j, int k)
 struct Ray {
     float o[3];      // segment origin
     float d[3];      // unit direction
-    float inv_d[3];  // 1 / d (0 where d == 0)
+    float inv_d[3];  // 1 / d (NaN where d == 0: no exit on that axis)
     int v[3];        // voxel of the current point
-    int lev;         // leaf size as a shift: the leaf spans 2^lev voxels per axis
+    int msk;         // leaf size - 1: the leaf spans msk + 1 = 2^shift voxels per axis (0: a voxel leaf)
     float M;         // leaf majorant (+ k_gas)
     float mn;        // leaf minorant (+ k_gas)
     float t;         // distance of the current point from o
@@ -159,11 +161,10 @@ struct Ray {
     uint32_t steps;  // leaves entered (guard)
 };
 
-// Voxel range [lo, hi] of the current leaf on axis a.
-__device__ __forceinline__ int leaf_lo(const Ray& R, int a) { return (R.v[a] >> R.lev) << R.lev; }
-__device__ __forceinline__ int leaf_hi(const DevScene& S, const Ray& R, int a)
+// Reciprocal of a direction component as the traversal wants it.
+__device__ __forceinline__ float dir_rcp(float d)
 {
-    return min(leaf_lo(R, a) + (1 << R.lev), S.n[a]) - 1;
+    return d != 0.0f ? __frcp_rn(d) : __int_as_float(0x7fffffff);
 }
 
 // Voxel of coordinate p on one axis: floor(p / h) by the rounded reciprocal,
@@ -176,6 +177,8 @@ __device__ __forceinline__ int locate(float p, float d, float h, float inv_h, in
 }
 
 // Leaf-map entry of the level-1 cell (of the tracked grid) holding voxel v.
+// The row index fits 32 bits: a row of level-1 cells holds at least 64 B of
+// bricks, leaf entries and octree cells, so 2^32 rows exceed the memory.
 __device__ __forceinline__ const uint2* leaf_entry(const DevScene& S, const int v[3])
 {
     const int b = S.lb;
@@ -187,40 +190,47 @@ __device__ __forceinline__ const uint2* leaf_entry(const DevScene& S, const int 
     }
     return S.leaf + ((size_t)(w[2] >> b) * S.nl[1] + (w[1] >> b)) * S.nl[0] + (w[0] >> b);
 #else
-    return S.leaf + ((size_t)(v[2] >> b) * S.nl[1] + (v[1] >> b)) * S.nl[0] + (v[0] >> b);
+    const uint32_t row = (uint32_t)(v[2] >> b) * (uint32_t)S.nl[1] + (uint32_t)(v[1] >> b);
+    return S.leaf + ((unsigned long long)row * (uint32_t)S.nl[0] + (uint32_t)(v[0] >> b));
+#endif
+}
+
+// Extinction of voxel v of brick `brick` (the voxel-leaf entry's first word).
+template <bool BF16>
+__device__ __forceinline__ float brick_fetch(const DevScene& S, uint32_t brick, const int v[3])
+{
+#ifdef MCRT_CHECKED
+    return kfetch<BF16>(S, v[0], v[1], v[2]);
+#else
+    const uint32_t off = ((((uint32_t)v[2] & 7u) << 3 | ((uint32_t)v[1] & 7u)) << 3) | ((uint32_t)v[0] & 7u);
+    const unsigned long long idx = (unsigned long long)brick * 512u + off;
+    if (BF16) return __uint_as_float((uint32_t)__ldg(S.vox16 + idx) << 16);
+    return __ldg(S.vox + idx);
 #endif
 }
 
 // Finish entering the leaf holding R.v from its leaf-map entry: size,
-// majorant and the exit distance / axis.
+// majorant and the exit distance / axis.  On each axis the exit face is the
+// upper one (min(lo + size, n)) when d > 0, else the lower one; an axis with
+// d == 0 has a NaN distance, which the minimum skips.
 template <bool BF16>
 __device__ __forceinline__ void finish_leaf(const DevScene& S, Ray& R, uint2 e)
 {
-    // entry: .x majorant bits, .y = minorant rounded down to bfloat16 | shift
-    R.lev = (int)(e.y & 0xFFFFu);
+    // entry: .x majorant bits (a voxel leaf: its brick), .y = minorant rounded down to bfloat16 | shift
+    R.msk = (int)((1u << (e.y & 31u)) - 1u);
     float M = __uint_as_float(e.x), mn = __uint_as_float(e.y & 0xFFFF0000u);
-    if (R.lev == 0) M = mn = kfetch<BF16>(S, R.v[0], R.v[1], R.v[2]);
+    if (R.msk == 0) M = mn = brick_fetch<BF16>(S, e.x, R.v);
     R.M = __fadd_rn(M, S.k_gas);
     R.mn = __fadd_rn(mn, S.k_gas);
-    const int s = R.lev;
     float ta[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int lo = (R.v[a] >> s) << s;
-        const int hi = min(lo + (1 << s), S.n[a]) - 1;
-        const float d = R.d[a];
-        if (d == 0.0f) {
-            ta[a] = __int_as_float(0x7f800000);
-        } else {
-            const int B = d > 0.0f ? hi + 1 : lo;
-            ta[a] = __fmul_rn(__fsub_rn(__fmul_rn(__int2float_rn(B), S.h[a]), R.o[a]), R.inv_d[a]);
-        }
+        const int up = min((R.v[a] | R.msk) + 1, S.n[a]);
+        const int B = R.d[a] > 0.0f ? up : (R.v[a] & ~R.msk);
+        ta[a] = __fmul_rn(__fsub_rn(__fmul_rn(__int2float_rn(B), S.h[a]), R.o[a]), R.inv_d[a]);
     }
-    int ax = 0;
-    float tm = ta[0];
-    if (ta[1] < tm) { ax = 1; tm = ta[1]; }
-    if (ta[2] < tm) { ax = 2; tm = ta[2]; }
-    R.ax = ax;
+    const float tm = fminf(fminf(ta[0], ta[1]), ta[2]);
+    R.ax = tm == ta[0] ? 0 : (tm == ta[1] ? 1 : 2);
     R.texit = fmaxf(tm, R.t);
 }
 
@@ -232,7 +242,7 @@ __device__ __forceinline__ void ray_begin(const DevScene& S, Ray& R, const float
     for (int a = 0; a < 3; ++a) {
         R.o[a] = p[a];
         R.d[a] = d[a];
-        R.inv_d[a] = (d[a] != 0.0f) ? __frcp_rn(d[a]) : 0.0f;
+        R.inv_d[a] = dir_rcp(d[a]);
         R.v[a] = locate(p[a], d[a], S.h[a], S.inv_h[a], 0, S.n[a] - 1);
     }
     R.t = 0.0f;
@@ -248,54 +258,42 @@ enum StepResult { kInside = 0, kTop = 1, kGround = 2 };
 // index instead steps across the face (hi + 1 or lo - 1).
 __device__ __forceinline__ void advance(const DevScene& S, const Ray& R, float tn, bool face, float p[3], int nv[3])
 {
-    const int s = R.lev;
-    int lo[3], hi[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
         p[b] = __fmaf_rn(tn, R.d[b], R.o[b]);
-        lo[b] = (R.v[b] >> s) << s;
-        hi[b] = min(lo[b] + (1 << s), S.n[b]) - 1;
-        nv[b] = locate(p[b], R.d[b], S.h[b], S.inv_h[b], lo[b], hi[b]);
-    }
-    // the exit axis steps across the face (its located value is discarded)
-    if (face) {
-        if (R.ax == 0) nv[0] = R.d[0] > 0.0f ? hi[0] + 1 : lo[0] - 1;
-        else if (R.ax == 1) nv[1] = R.d[1] > 0.0f ? hi[1] + 1 : lo[1] - 1;
-        else nv[2] = R.d[2] > 0.0f ? hi[2] + 1 : lo[2] - 1;
+        const int lo = R.v[b] & ~R.msk;
+        const int hi = min(R.v[b] | R.msk, S.n[b] - 1);
+        nv[b] = locate(p[b], R.d[b], S.h[b], S.inv_h[b], lo, hi);
+        // the exit axis steps across the face (its located value is discarded)
+        const int across = R.d[b] > 0.0f ? hi + 1 : lo - 1;
+        const bool exits = face && R.ax == b;
+        nv[b] = exits ? across : nv[b];
     }
 }
 
 // Complete a face crossing prepared by advance(face = true): the ground or
 // the top, or the periodic wrap of x / y (the segment then restarts on the
 // face: o on the face exactly, t = 0, *wrapped_dt = distance of the finished
-// segment), then the new voxel.  The caller loads the leaf-map entry of R.v
-// and calls finish_leaf when the result is kInside.
+// segment), then the new voxel.  Only the exit axis can leave the domain.
+// The caller loads the leaf-map entry of R.v and calls finish_leaf when the
+// result is kInside.
 __device__ __forceinline__ int cross_face(const DevScene& S, Ray& R, const float p[3], int nv[3], float* wrapped_dt)
 {
-    const int ax = R.ax;
-    const float te = R.texit;
     *wrapped_dt = 0.0f;
-    R.t = te;
-    if (ax == 2) {
+    R.t = R.texit;
+    if ((uint32_t)nv[0] >= (uint32_t)S.n[0] || (uint32_t)nv[1] >= (uint32_t)S.n[1] ||
+        (uint32_t)nv[2] >= (uint32_t)S.n[2]) {
         if (nv[2] < 0) return kGround;
         if (nv[2] >= S.n[2]) return kTop;
-    } else {
-        int wrapped = 0;
+        *wrapped_dt = R.texit;
+        R.o[2] = p[2];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            if (b != ax) continue;
-            if (nv[b] < 0) { nv[b] = S.n[b] - 1; wrapped = 1; }
-            else if (nv[b] >= S.n[b]) { nv[b] = 0; wrapped = 2; }
+            R.o[b] = p[b];
+            if (nv[b] < 0) { nv[b] = S.n[b] - 1; R.o[b] = S.Lper[b]; }
+            else if (nv[b] >= S.n[b]) { nv[b] = 0; R.o[b] = 0.0f; }
         }
-        if (wrapped) {
-            *wrapped_dt = te;
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                R.o[b] = p[b];
-                if (b == ax) R.o[b] = (wrapped == 1) ? (b == 0 ? S.Lper[0] : S.Lper[1]) : 0.0f;
-            }
-            R.t = 0.0f;
-        }
+        R.t = 0.0f;
     }
     R.v[0] = nv[0]; R.v[1] = nv[1]; R.v[2] = nv[2];
     ++R.steps;
@@ -453,7 +451,7 @@ __device__ __forceinline__ float hf_height(const DevScene& S, float x, float y, 
 {
     const float fx = x * S.inv_hc[0], fy = y * S.inv_hc[1];
     const int i = __float2int_rd(fx), j = __float2int_rd(fy);
-    const float u = fx - (float)i, v = fy - (float)j;
+    const float u = __fmaf_rn(x, S.inv_hc[0], -(float)i), v = __fmaf_rn(y, S.inv_hc[1], -(float)j);
     float hc4[4];
     hf_corners(S, i, j, hc4);
     float a, b, c;

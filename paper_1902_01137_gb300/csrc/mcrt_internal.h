@@ -199,10 +199,14 @@ struct TraceParams {
     const volatile int* cancel;
 };
 
-// Rare phases (path start, ray start, vertex) of a warp run once this many
-// of its lanes wait for them (the default when a caller passes 0), or when
-// fewer than 33 - that many lanes are stepping.  Launch shape only.
-constexpr int kDefaultRareBatch = 10;
+// A warp leaves its step loop for a rare pass (path starts, ray starts,
+// vertices, ended rays) once this many of its lanes wait for one (the default
+// when a caller passes 0).  Launch shape only.  A pass costs about three step
+// iterations whatever its lane count, so waiting pays until the step loop
+// runs half empty: cumulus image of 16.8 M paths 62.1, 57.3, 56.3, 57.9,
+// 64.2 ms at 8, 12, 16, 20, 24 lanes; flux of the same field 53.3, 51.7,
+// 49.9, 48.3, 52.1 ms; octree image 35.2, 32.8, 32.3, 32.9, 35.3 ms.
+constexpr int kDefaultRareBatch = 16;
 inline void set_rare_batch(TraceParams& P, int requested)
 {
     P.rare_batch = requested > 0 ? requested : kDefaultRareBatch;
@@ -239,8 +243,14 @@ cudaError_t launch_finalize(const double* s1, const double* s2, double n, int co
 // Thresholds from GB300 measurements on the cumulus field: chunk 1 below
 // 48 paths per lane, 2 below 160, 4 below 400, else 8 (the most the FP32
 // chunk sums are bounded for); camera chunks divide spp.
-inline uint32_t auto_chunk(unsigned long long total, unsigned long long lanes, uint32_t spp)
+// A chunk's sums are rounded to FP32, so the rule goes by the request alone:
+// lanes are those of the given grid, or of 28 warps per SM, whatever the
+// kernel's occupancy.
+inline uint32_t auto_chunk(unsigned long long total, int sm_count, int grid_size, int block, uint32_t spp)
 {
+    const unsigned long long lanes =
+        (grid_size ? (unsigned long long)grid_size : (unsigned long long)sm_count * (unsigned)(28 / (block / 32))) *
+        (unsigned)block;
     const double per_lane = lanes ? (double)total / (double)lanes : 0.0;
     uint32_t c = per_lane < 48.0 ? 1u : (per_lane < 160.0 ? 2u : (per_lane < 400.0 ? 4u : 8u));
     if (spp) {

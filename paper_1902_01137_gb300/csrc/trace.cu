@@ -1,14 +1,16 @@
 // trace.cu -- persistent path-tracing kernel (sm_103a).
 //
-// One GPU thread carries one path at a time; its state (traversal, weights,
-// the two Philox draw sequences) lives in registers.  Every loop iteration
-// advances each live lane by exactly one traversal step -- either one leaf
-// crossed or one tentative collision handled -- whatever ray it is on (the
-// path's free flight or a sun ray), so all lanes of a warp run the same code
-// and divergence is limited to the short event-handling branches.  Lanes
-// whose chunk of paths is done are refilled at the top of the loop: the warp
-// ballots its idle lanes and claims new path ids for all of them with one
-// atomic (work stays balanced to the last paths).
+// One GPU thread carries one path at a time.  What a traversal step needs
+// lives in registers (the ray, its leaf, the optical depth left); the rest of
+// the path (weights, vertex, directions, ids, sums) in a shared-memory slot
+// of its own, touched only when a ray starts or ends.  A warp alternates
+// between two loops:
+//   steps  every lane on a ray crosses one leaf or handles one tentative
+//          collision per iteration, whatever ray it is on (the path's free
+//          flight or a sun ray), until enough lanes wait for something else;
+//   rare   one pass over all waiting lanes: rays and paths that ended, chunk
+//          sums, new chunks (one atomic per warp), the one Philox block,
+//          path starts, vertices, ray starts.
 //
 // Physics (Villefranque et al. 2019):
 //   free flight: null-collision sampling over leaves of uniform majorant M
@@ -32,19 +34,23 @@
 // first optical depth), a Rayleigh vertex its species from word 0 of block
 // kBlockVertex.
 //
-// Loop structure (one iteration): flush finished chunks and claim new ones
-// (convergent); one Philox block per lane; one phase of work per lane (path
-// start, traversal step, vertex, ray start -- a camera path start or a
-// vertex, learned or not, goes on into the ray start it sets up, whose first
-// optical depth is a word of the block already drawn); one 8-byte load (the
-// voxel of a tentative collision or the leaf-map entry of the leaf entered);
-// the leaf set-up; the end of a ray or path.
+// What bounds it: instruction issue.  The split keeps the step loop short
+// (no random block, sums, claims or path state in it) and its registers few
+// enough for 8 blocks of 128 threads an SM without spills; a single loop
+// with everything in it, at 72 registers and one Philox block per iteration,
+// took 95.2 ms for 16.8 M paths of the 512 x 512 x 160 cumulus image, this
+// one 56.3 ms (octree image of 11.8 M paths 46.5 -> 32.3 ms, 16.8 M flux
+// paths 81.6 -> 49.9 ms, 4 M over a relief 45.7 -> 25.4 ms).  7, 9 and 10
+// resident blocks: 56.7, 56.9 and 57.0 ms.
+// A step draws its Philox block only when its result depends on it: a
+// voxel leaf's majorant is the voxel itself, so a tentative collision there
+// is real (a sun ray's ratio 1 - k/M is 0) whatever the draw.
 #include <cuda_bf16.h>
 
 #include "mcrt_internal.h"
 
 #ifndef MCRT_TRACE_MIN_BLOCKS
-#define MCRT_TRACE_MIN_BLOCKS 7   // resident blocks of 128 threads the register budget must allow (72 registers)
+#define MCRT_TRACE_MIN_BLOCKS 8   // resident blocks of 128 threads the register budget must allow (64 registers)
 #endif
 
 namespace mcrt {
@@ -67,24 +73,46 @@ constexpr int kCounters = 10;
 // work queue ran dry, [12] longest time (ns) a warp ran in total.
 enum { C_MAX_ITERS = 10, C_T_DRY = 11, C_T_END = 12 };
 // Counting mode also records, per warp, the SM clock cycles spent in each
-// section of the loop body (slots 13..21): loop top, Philox, path start,
-// ray start, step, vertex, load, after-load, ray/path end.
+// section of the loop (slots 13..21): sums and claims, Philox, path start,
+// ray start, steps, vertex, (two unused,) ended rays and paths.
 constexpr int C_SEC = 13;
 constexpr int kSections = 9;
-// ... and, per warp iteration, lane occupancy (slots 22..29): iterations,
-// lanes holding a path, stepping, at a tentative collision, running a rare
-// phase, waiting for one, iterations that ran rare phases, lanes without a path.
+// ... and, per step iteration, lane occupancy (slots 22..29): iterations,
+// lanes holding a path, stepping, at a tentative collision, running in a rare
+// pass, waiting for one, rare passes, lanes without a path.
 constexpr int C_OCC = 22;
 constexpr int kOcc = 8;
 
-// Each lane is in one phase per iteration: it starts a path, starts a ray
-// (flight or sun ray), takes one traversal step, or handles the vertex that
-// ended a flight.  Every lane evaluates one Philox block per iteration at
-// one site, whose counter depends on the phase (a camera path start or a
-// vertex that continues into its ray start takes that ray's first optical
-// depth from a word of it); the voxel / leaf-entry load and the leaf set-up
-// also run at one site each.
-enum Phase { PH_IDLE = 0, PH_START, PH_BEGIN, PH_STEP, PH_VERTEX, PH_RESUME, PH_TERRAIN };
+// What a lane is doing.  PH_STEP lanes take traversal steps; every other
+// phase but PH_IDLE waits for the warp's next rare pass.
+enum Phase {
+    PH_STEP = 0,
+    PH_IDLE,        // no chunk, nothing left to claim
+    PH_CLAIM,       // no chunk
+    PH_FLUSH,       // chunk finished: its sums go to the tally, then a new chunk
+    PH_START,       // a path starts
+    PH_BEGIN,       // a ray starts: the flight from the vertex, or a flux path's direct sun ray
+    PH_VERTEX,      // a volume vertex
+    PH_GROUND,      // a ground vertex
+    PH_RESUME,      // a path stopped at a learned vertex goes on
+    PH_SUSPEND,     // a path stops at a learned vertex
+    PH_TERRAIN,     // a flight reached the relief layer: find its ground hit
+    PH_SUN_END,     // a sun ray ended with transmissivity Ts
+    PH_END          // the path ends
+};
+
+// Per-thread slots of a path's state outside its registers, [field][thread]
+// (conflict-free); fields past kCold depend on the kernel variant.
+enum Cold {
+    K_PID_LO = 0, K_PID_HI, K_LEFT,          // path id, paths left in the chunk (this one included)
+    K_CELL,                                  // tally cell (pixel; batch item)
+    K_EV,                                    // event index | kTermAfter
+    K_W, K_SCORE, K_CF,                      // weight, score so far, factor of the sun ray's estimate
+    K_VX, K_VY, K_VZ, K_VK,                  // vertex and its extinction
+    K_NX, K_NY, K_NZ,                        // direction of the next flight
+    kCold
+};
+constexpr uint32_t kTermAfter = 0x80000000u;   // the path ends with this event's estimate
 
 // EXTRA: the variants that also handle decomposition tracking of sun rays
 // and Rayleigh clear air (chosen at run time); the others carry neither, so
@@ -96,38 +124,54 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
 {
     // quantities per path: camera radiance; flux T_dir, T_dif, T_tot (+ dT/dg, dT/dalpha in batches)
     constexpr int NQ = (SENSOR == kCamera) ? 1 : (BATCH ? 5 : 3);
-    const int lane = threadIdx.x & 31;
-    const unsigned lt_mask = (1u << lane) - 1u;
-
-    // ---- per-lane state ------------------------------------------------------
-    unsigned long long pid = 0, pend = 0;   // current path, end of the lane's chunk
-    bool chunk = false;                     // the lane holds a chunk
-    bool exhausted = false;                 // warp-uniform: nothing left to claim
-    int phase = PH_IDLE;
-    unsigned cell = 0;                      // tally cell of the chunk
-    int px = 0, py = 0;                     // camera pixel of the chunk
+    // decomposition tracking needs the leaf minorants
+    constexpr bool DECOMP = EXTRA && !BATCH;
     // chunk sums of x and x^2 in FP32 (a chunk is at most 8 paths: relative
     // error below 7 * 2^-24 of the sum of |x| before the FP64 atomic add)
-    float acc[2 * NQ];
-#pragma unroll
-    for (int q = 0; q < 2 * NQ; ++q) acc[q] = 0.0f;
+    constexpr int K_ACC = kCold;
+    constexpr int K_TDIR = K_ACC + 2 * NQ;                     // flux: direct transmissivity
+    constexpr int K_FZ = K_TDIR + (SENSOR == kFlux ? 1 : 0);   // heightfield flux: n_z of the surface at the path start
+    constexpr int K_SG = K_FZ + (TERRAIN ? 1 : 0);             // batches: d/dg ...
+    constexpr int K_SVP = K_SG + 1, K_CFS = K_SG + 2, K_DSC = K_SG + 3;
+    constexpr int K_SA = K_SG + 4, K_DAL = K_SG + 5;           // ... and d/dalpha, the droplets' absorptivity
+    constexpr int K_LV = K_SG + (BATCH ? 6 : 0);               // learned mode: volume vertices so far,
+    constexpr int K_REC = K_LV + 1;                            // training record awaiting its own estimate
+    constexpr int kFields = K_LV + (LEARNED ? 2 : 0);
+    __shared__ float cold[kFields][128];
+
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int tid = threadIdx.x;
+    auto F = [&](int f) -> float& { return cold[f][tid]; };
+    auto geti = [&](int f) -> uint32_t { return __float_as_uint(cold[f][tid]); };
+    auto seti = [&](int f, uint32_t v) { cold[f][tid] = __uint_as_float(v); };
+    auto get_pid = [&]() -> unsigned long long {
+        return (unsigned long long)geti(K_PID_LO) | ((unsigned long long)geti(K_PID_HI) << 32);
+    };
+    auto set_pid = [&](unsigned long long pid) {
+        seti(K_PID_LO, (uint32_t)pid);
+        seti(K_PID_HI, (uint32_t)(pid >> 32));
+    };
+
+    // ---- per-lane state ------------------------------------------------------
+    const float kInf = __int_as_float(0x7f800000);
+    bool exhausted = false;                 // warp-uniform: nothing left to claim
+    int phase = PH_CLAIM;
     Ray R;
     int kind = kMain;
-    uint32_t c2 = 0, blk = 1, ev = 0;
-    float tau = 0.0f, Ts = 1.0f, w = 1.0f, score = 0.0f, cf = 0.0f, tdir = 0.0f;
-    bool term_after = false, vground = false;
-    float vk = 0.0f;                        // extinction at the vertex
-    uint32_t lv = 0;                        // volume vertices so far (learned mode)
-    uint32_t cur_rec = 0xFFFFFFFFu;         // training record awaiting its own estimate
-    bool suspend = false;                   // stop this path until the network has run
-    float tg = __int_as_float(0x7f800000);  // heightfield: distance of the flight's ground hit from R.o
-    float tpend = __int_as_float(0x7f800000);   // heightfield: where the flight enters the relief layer (walk pending)
-    float fz = 1.0f;                        // heightfield flux: n_z of the surface at the path start
-    float vx[3] = {0.0f, 0.0f, 0.0f}, nd[3] = {0.0f, 0.0f, 1.0f};
+    uint32_t blk = 1;                       // Philox block of the ray's next tentative collision
+    float tau = 0.0f, Ts = 1.0f;
+    float tg = kInf;                        // heightfield: distance of the flight's ground hit from R.o
+    float tpend = kInf;                     // heightfield: where the flight enters the relief layer (walk pending)
+#pragma unroll
+    for (int q = 0; q < 2 * NQ; ++q) F(K_ACC + q) = 0.0f;
+    seti(K_CELL, 0u);
+    seti(K_LEFT, 0u);
+    if (LEARNED) seti(K_REC, 0xFFFFFFFFu);
     unsigned long long cnt[kCounters];
 #pragma unroll
     for (int q = 0; q < kCounters; ++q) cnt[q] = 0;
-    uint32_t path_iters = 0, max_iters = 0;
+    uint32_t path_iters = 0, max_iters = 0, tents = 0;
     unsigned long long sec[kSections];
 #pragma unroll
     for (int q = 0; q < kSections; ++q) sec[q] = 0;
@@ -143,58 +187,178 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
             tclk = now;
         }
     };
-    int item = 0;                           // batch item of the lane's chunk
-    uint2 rkey = P.key;                     // Philox key of that item
-    float sg = 0.0f, sv_pending = 0.0f, cfs = 0.0f, dscore = 0.0f;   // d/dg (batches)
-    float sa = 0.0f, dal = 0.0f;            // d/dalpha, the droplets' absorptivity (batches)
     uint64_t t_start = 0, t_dry = 0;
     if (P.deadline_ns || COUNT) t_start = globaltimer_ns();
-    uint32_t iter = 0;
+    int budget = 1024;                      // step iterations until the next deadline / cancel check
 
     for (;;) {
+        // ==== rare pass: every lane that is not stepping ======================
+        // ---- rays and paths that ended ---------------------------------------
+        if (phase == PH_SUN_END) {
+            if (SENSOR == kFlux && kind == kSunDirect) {
+                if constexpr (SENSOR == kFlux) F(K_TDIR) = TERRAIN ? F(K_TDIR) * Ts : Ts;
+                seti(K_EV, 0u);
+                kind = kMain;
+                phase = PH_BEGIN;
+            } else {
+                const float cf = F(K_CF);
+                F(K_SCORE) += cf * Ts;
+                if constexpr (BATCH) {
+                    F(K_DSC) += cf * Ts * (F(K_SG) + F(K_CFS));
+                    if (EXTRA) F(K_DAL) += cf * Ts * F(K_SA);
+                    F(K_SG) += F(K_SVP);
+                }
+                if constexpr (LEARNED) {
+                    const uint32_t rec = geti(K_REC);
+                    if (rec != 0xFFFFFFFFu) {
+                        P.rec_val[4 * (size_t)rec + 2] = cf * Ts;
+                        seti(K_REC, 0xFFFFFFFFu);
+                    }
+                }
+                const uint32_t e = geti(K_EV);
+                if (e & kTermAfter) {
+                    phase = PH_END;
+                } else {
+                    seti(K_EV, e + 1u);
+                    kind = kMain;
+                    phase = PH_BEGIN;
+                }
+            }
+        }
+        if (phase == PH_END) {
+            const float score = F(K_SCORE);
+            if constexpr (SENSOR == kCamera) {
+                F(K_ACC) += score;
+                F(K_ACC + 1) += score * score;
+            } else {
+                const float tdir = F(K_TDIR);
+                const DevScene& S = BATCH ? P.items[geti(K_CELL)].S : P.S;
+                const float pi_over_mu0 = __fdividef(kPi, TERRAIN ? F(K_FZ) * S.sun[2] : S.sun[2]);
+                const float tf = pi_over_mu0 * score;
+                const float tt = tdir + tf;
+                F(K_ACC + 0) += tdir; F(K_ACC + 1) += tdir * tdir;
+                F(K_ACC + 2) += tf; F(K_ACC + 3) += tf * tf;
+                F(K_ACC + 4) += tt; F(K_ACC + 5) += tt * tt;
+                if constexpr (BATCH) {
+                    const float dt = pi_over_mu0 * F(K_DSC);
+                    F(K_ACC + 6) += dt; F(K_ACC + 7) += dt * dt;
+                    if (EXTRA) {
+                        const float da = pi_over_mu0 * F(K_DAL);
+                        F(K_ACC + 8) += da; F(K_ACC + 9) += da * da;
+                    }
+                }
+            }
+            if (COUNT) {
+                cnt[C_PATHS]++;
+                max_iters = max(max_iters, path_iters);
+            }
+            const unsigned long long pid = get_pid();
+            if (LEARNED && P.final_score) P.final_score[pid - P.path_base] = score;
+            const uint32_t left = geti(K_LEFT) - 1u;
+            seti(K_LEFT, left);
+            set_pid(pid + 1u);
+            phase = left ? PH_START : PH_FLUSH;
+        }
+        mark(8);
+        // ---- stop paths at a learned vertex: state and features to the queue
+        if constexpr (LEARNED) {
+            const unsigned smask = __ballot_sync(kFull, phase == PH_SUSPEND);
+            if (smask) {
+                const int leader = __ffs(smask) - 1;
+                unsigned base = 0;
+                if (lane == leader) base = atomicAdd(P.qout_count, (unsigned)__popc(smask));
+                base = __shfl_sync(kFull, base, leader);
+                if (phase == PH_SUSPEND) {
+                    const DevScene& S = P.S;
+                    const unsigned slot = base + (unsigned)__popc(smask & lt_mask);
+                    const unsigned long long pid = get_pid();
+                    if (slot < P.qout_cap) {
+                        // features: position in [-1, 1], incoming direction, ln(k), ln(M1), ln(M2)
+                        const float vx[3] = {F(K_VX), F(K_VY), F(K_VZ)}, vk = F(K_VK);
+                        const int nv[3] = {R.v[0], R.v[1], R.v[2]};   // (the collision's voxel)
+                        const float Lz = (float)S.n[2] * S.h[2];
+                        float f[9];
+                        f[0] = 2.0f * vx[0] / S.Lper[0] - 1.0f;
+                        f[1] = 2.0f * vx[1] / S.Lper[1] - 1.0f;
+                        f[2] = 2.0f * vx[2] / Lz - 1.0f;
+                        f[3] = R.d[0]; f[4] = R.d[1]; f[5] = R.d[2];
+                        f[6] = logf(vk + 1e-6f);
+                        const float M1 = __ldg(P.pyr1 + ((size_t)(nv[2] >> 3) * P.d1[1] + (nv[1] >> 3)) * P.d1[0] +
+                                               (nv[0] >> 3));
+                        const int s2 = 3 * P.lev2;
+                        const float M2 = __ldg(P.pyr2 + ((size_t)(nv[2] >> s2) * P.d2[1] + (nv[1] >> s2)) * P.d2[0] +
+                                               (nv[0] >> s2));
+                        f[7] = logf(M1 + S.k_gas + 1e-6f);
+                        f[8] = logf(M2 + S.k_gas + 1e-6f);
+                        uint32_t pk[8];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const __nv_bfloat162 v = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+                            pk[i] = *reinterpret_cast<const uint32_t*>(&v);
+                        }
+                        pk[4] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f[8]));
+                        pk[5] = pk[6] = pk[7] = 0u;
+                        P.qout_feat[2 * (size_t)slot] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        P.qout_feat[2 * (size_t)slot + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        P.qout[4 * (size_t)slot] = make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), geti(K_EV), geti(K_LV));
+                        P.qout[4 * (size_t)slot + 1] = make_uint4(__float_as_uint(vx[0]), __float_as_uint(vx[1]),
+                                                                  __float_as_uint(vx[2]), __float_as_uint(vk));
+                        P.qout[4 * (size_t)slot + 2] = make_uint4(__float_as_uint(R.d[0]), __float_as_uint(R.d[1]),
+                                                                  __float_as_uint(R.d[2]), geti(K_W));
+                        P.qout[4 * (size_t)slot + 3] =
+                            make_uint4(geti(K_SCORE), SENSOR == kFlux ? geti(K_TDIR) : 0u, 0u, 0u);
+                    }
+                    const uint32_t left = geti(K_LEFT) - 1u;
+                    seti(K_LEFT, left);
+                    set_pid(pid + 1u);
+                    phase = left ? PH_START : PH_FLUSH;
+                }
+            }
+        }
         // ---- flush finished chunks: lanes sharing a cell are summed first --
-        bool pending = chunk && phase == PH_IDLE;
-        if (pending) chunk = false;
-        unsigned fmask = __ballot_sync(kFull, pending);
+        unsigned fmask = __ballot_sync(kFull, phase == PH_FLUSH);
         while (fmask) {
             const int src = __ffs(fmask) - 1;
-            const unsigned c = __shfl_sync(kFull, cell, src);
+            const unsigned my = geti(K_CELL);
+            const unsigned c = __shfl_sync(kFull, my, src);
             MCRT_CHECK(c < (SENSOR == kCamera ? (unsigned)(P.width * P.height) : (BATCH ? (unsigned)P.n_items : 1u)), 3);
-            const bool mine = pending && cell == c;
+            const bool mine = phase == PH_FLUSH && my == c;
 #pragma unroll
             for (int q = 0; q < 2 * NQ; ++q) {
-                double a = mine ? (double)acc[q] : 0.0;
+                double a = mine ? (double)F(K_ACC + q) : 0.0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
                 if (lane == src) atomicAdd(((q & 1) ? P.s2 : P.s1) + (size_t)c * NQ + (q >> 1), a);
             }
             if (mine) {
-                pending = false;
+                phase = PH_CLAIM;
 #pragma unroll
-                for (int q = 0; q < 2 * NQ; ++q) acc[q] = 0.0f;
+                for (int q = 0; q < 2 * NQ; ++q) F(K_ACC + q) = 0.0f;
             }
-            fmask = __ballot_sync(kFull, pending);
+            fmask = __ballot_sync(kFull, phase == PH_FLUSH);
         }
         // ---- claim chunks for idle lanes (one atomic per warp) -------------
-        const unsigned idle = __ballot_sync(kFull, !chunk);
-        if (idle && !exhausted) {
-            const int nidle = __popc(idle);
-            const int leader = __ffs(idle) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(&P.work->next, (unsigned long long)nidle * P.chunk);
-            base = __shfl_sync(kFull, base, leader);
-            if (base + (unsigned long long)nidle * P.chunk >= P.total) {
-                exhausted = true;
-                if (COUNT) t_dry = globaltimer_ns();
+        const unsigned idle = __ballot_sync(kFull, phase == PH_CLAIM);
+        if (idle) {
+            unsigned long long base = P.total;
+            if (!exhausted) {
+                const int nidle = __popc(idle);
+                const int leader = __ffs(idle) - 1;
+                if (lane == leader) base = atomicAdd(&P.work->next, (unsigned long long)nidle * P.chunk);
+                base = __shfl_sync(kFull, base, leader);
+                if (base + (unsigned long long)nidle * P.chunk >= P.total) {
+                    exhausted = true;
+                    if (COUNT) t_dry = globaltimer_ns();
+                }
             }
-            if (!chunk) {
-                pid = base + (unsigned long long)__popc(idle & lt_mask) * P.chunk;
+            if (phase == PH_CLAIM) {
+                phase = PH_IDLE;
+                unsigned long long pid = base + (unsigned long long)__popc(idle & lt_mask) * P.chunk;
                 if (pid < P.total) {
-                    pend = min(pid + (unsigned long long)P.chunk, P.total);
-                    chunk = true;
+                    uint32_t left = (uint32_t)min((unsigned long long)P.chunk, P.total - pid);
                     phase = (LEARNED && P.resume) ? PH_RESUME : PH_START;
                     // the batch (learned mode) or shard (flux) this launch traces
-                    if (!BATCH && !(LEARNED && P.resume)) { pid += P.path_base; pend += P.path_base; }
+                    if (!BATCH && !(LEARNED && P.resume)) pid += P.path_base;
                     if constexpr (BATCH) {
                         // items own chunk-aligned id ranges: find the item, use its local ids
                         int lo = 0, hi = P.n_items - 1;
@@ -203,12 +367,11 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                             if (P.items[mid].begin <= pid) lo = mid;
                             else hi = mid - 1;
                         }
-                        item = lo;
                         const unsigned long long b = P.items[lo].begin, np = P.items[lo].npaths;
                         pid -= b;
-                        pend = min(pend - b, np);
-                        rkey = P.items[lo].key;
-                        if (pid >= np) { chunk = false; phase = PH_IDLE; }
+                        if (pid >= np) phase = PH_CLAIM;      // padding ids of the item's last chunk
+                        else left = (uint32_t)min((unsigned long long)left, np - pid);
+                        seti(K_CELL, (uint32_t)lo);
                     }
                     if constexpr (SENSOR == kCamera) {
                         unsigned long long pix = pid / P.spp;
@@ -218,96 +381,78 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                             // its result do not depend on the order
                             const unsigned long long off = pid - pix * P.spp;
                             pix = __ldg(P.pix_order + pix);
-                            pid = pix * P.spp + off;
-                            pend = pid + P.chunk;          // a chunk never straddles two pixels
+                            pid = pix * P.spp + off;          // a chunk never straddles two pixels
                         }
-                        cell = (unsigned)pix;
-                        px = (int)(pix % (unsigned long long)P.width);
-                        py = (int)(pix / (unsigned long long)P.width);
-                    } else {
-                        cell = BATCH ? (unsigned)item : 0u;
+                        seti(K_CELL, (uint32_t)pix);
                     }
+                    set_pid(pid);
+                    seti(K_LEFT, left);
                 }
             }
         }
-        if (!__any_sync(kFull, chunk)) break;
-        // ---- deadline / cancel, every 1024 iterations ------------------------
-        if ((++iter & 1023u) == 0 && (P.deadline_ns || P.cancel)) {
-            int stop = 0;
-            if (lane == 0) {
-                if (P.cancel && *P.cancel) stop = 2;
-                else if (P.deadline_ns && globaltimer_ns() - t_start > P.deadline_ns) stop = 1;
-                const int others = *reinterpret_cast<volatile int*>(&P.work->status);
-                if (others) stop = others;
-            }
-            stop = __shfl_sync(kFull, stop, 0);
-            if (stop) {
-                if (lane == 0) atomicMax(&P.work->status, stop);
-                break;
+        const unsigned live = __ballot_sync(kFull, phase != PH_IDLE);
+        if (!live) break;
+        // ---- deadline / cancel, every 1024 step iterations --------------------
+        if (budget <= 0) {
+            budget = 1024;
+            if (P.deadline_ns || P.cancel) {
+                int stop = 0;
+                if (lane == 0) {
+                    if (P.cancel && *P.cancel) stop = 2;
+                    else if (P.deadline_ns && globaltimer_ns() - t_start > P.deadline_ns) stop = 1;
+                    const int others = *reinterpret_cast<volatile int*>(&P.work->status);
+                    if (others) stop = others;
+                }
+                stop = __shfl_sync(kFull, stop, 0);
+                if (stop) {
+                    if (lane == 0) atomicMax(&P.work->status, stop);
+                    break;
+                }
             }
         }
-        if (COUNT && phase != PH_IDLE) ++path_iters;
-        if (COUNT) { __syncwarp(); tclk = clock64(); }
-
-        // ---- rare phases (path start, ray start, vertex) run in batches: a
-        //      lane waits until enough lanes of its warp need one, or until
-        //      few lanes are stepping ------------------------------------------
-        // (heightfield: a flight whose current leaf reaches down into the relief
-        //  layer first finds its ground hit, a rare phase of its own)
-        if (TERRAIN && phase == PH_STEP && R.texit >= tpend) phase = PH_TERRAIN;
-        const bool rare = phase == PH_START || phase == PH_BEGIN || phase == PH_VERTEX || phase == PH_RESUME ||
-                          (TERRAIN && phase == PH_TERRAIN);
-        const unsigned rare_mask = __ballot_sync(kFull, rare);
-        const unsigned step_mask = __ballot_sync(kFull, phase == PH_STEP);
-        const bool run_rare = __popc(rare_mask) >= P.rare_batch || __popc(step_mask) < P.min_steppers;
-        // every rare kind runs in the same iteration: path starts and
-        // vertices (learned ones resumed too) go on into their ray start, and
-        // ground walks start there as well, so the ray-start and walk
-        // branches execute once with all their lanes
-        const int ph = (phase == PH_STEP || (rare && run_rare)) ? phase : PH_IDLE;
-
-        // ---- the scene of the lane's chunk (one per batch item) ---------------
-        const DevScene& S = BATCH ? P.items[item].S : P.S;
-
-        // ---- the one Philox block of this iteration ---------------------------
-        const float seg = (TERRAIN ? fminf(R.texit, tg) : R.texit) - R.t;
-        // tracking majorant: the leaf's M, or M - m for a sun ray in
-        // decomposition tracking (the minorant m is applied exactly)
-        const bool decomp = EXTRA && kind != kMain && P.sun_mode == MCRT_SUN_DECOMP;
-        const float Mt = decomp ? R.M - R.mn : R.M;
-        const float Mseg = Mt * seg;
-        const bool tent = ph == PH_STEP && Mt > 0.0f && tau < Mseg;
+        const bool ran = phase != PH_STEP && phase != PH_IDLE;
         if (COUNT) {
-            const unsigned busy = __ballot_sync(kFull, chunk), tm = __ballot_sync(kFull, tent);
-            const unsigned rr = __ballot_sync(kFull, rare && ph != PH_IDLE);
-            occ[0] += 1; occ[1] += __popc(busy); occ[2] += __popc(step_mask); occ[3] += __popc(tm);
-            occ[4] += __popc(rr); occ[5] += __popc(rare_mask) - __popc(rr); occ[6] += rr ? 1 : 0;
-            occ[7] += 32 - __popc(busy);
+            if (ran) ++path_iters;
+            const unsigned rr = __ballot_sync(kFull, ran);
+            occ[4] += __popc(rr);
+            occ[6] += rr ? 1 : 0;
+            __syncwarp();
         }
-        uint32_t xc2 = c2, xblk = 0u;
-        if (ph == PH_START) xc2 = 2u;
-        else if (ph == PH_STEP) xblk = blk;
-        else if (ph == PH_VERTEX) { xc2 = (ev << 2) | 1u; xblk = 0u; }   // the sun ray's block 0
         mark(0);
-        const uint4 x = draw_block(pid, xc2, xblk, rkey);
-        mark(1);
 
-        // ---- phase work before the load ---------------------------------------
-        int evc = EV_NONE;
-        float p[3];
-        int nv[3] = {0, 0, 0};
-        const uint2* ptr = nullptr;
-        uint32_t sub = 0;
-        int st = kInside;
-        bool setup = false;          // enter a leaf after the load
-        bool walk = false;           // heightfield: find this ray's ground hit now
-        bool merge = false;          // a path start or vertex whose ray starts in this iteration too
-        uint32_t mword = 0u;         // ... the word giving that ray's first optical depth
-        if (ph == PH_START) {
-            w = 1.0f; score = 0.0f; ev = 0; tdir = 0.0f; term_after = false;
-            if (BATCH) { sg = 0.0f; sv_pending = 0.0f; cfs = 0.0f; dscore = 0.0f; sa = 0.0f; dal = 0.0f; }
-            if (COUNT) path_iters = 0;
+        // ---- the one Philox block of this pass ---------------------------------
+        const DevScene& S = BATCH ? P.items[geti(K_CELL)].S : P.S;
+        const bool vert = phase == PH_VERTEX || phase == PH_GROUND;
+        const uint32_t ev = geti(K_EV);
+        const unsigned long long pid = get_pid();
+        const uint2 rkey = BATCH ? P.items[geti(K_CELL)].key : P.key;
+        bool begin = phase == PH_BEGIN;   // start a ray now ...
+        uint32_t tw = 0u;                 // ... whose first optical depth comes from this word
+        bool walk = false;                // heightfield: find this ray's ground hit now
+        float vx[3] = {0.0f, 0.0f, 0.0f}, nd[3] = {0.0f, 0.0f, 0.0f};
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (ran) {
+            uint32_t xc2 = kind == kSunDirect ? 3u : ev << 2;     // PH_BEGIN: the ray's own block 0
+            if (phase == PH_START) xc2 = 2u;
+            else if (vert) xc2 = (ev << 2) | 1u;                   // the sun ray's block 0
+            x = draw_block(pid, xc2, 0u, rkey);
+            tw = x.x;
+            vx[0] = F(K_VX); vx[1] = F(K_VY); vx[2] = F(K_VZ);
+            nd[0] = F(K_NX); nd[1] = F(K_NY); nd[2] = F(K_NZ);
+        }
+        mark(1);
+        if (phase == PH_START) {
+            seti(K_EV, 0u);
+            F(K_W) = 1.0f;
+            F(K_SCORE) = 0.0f;
+            if constexpr (BATCH) {
+                F(K_SG) = 0.0f; F(K_SVP) = 0.0f; F(K_CFS) = 0.0f; F(K_DSC) = 0.0f; F(K_SA) = 0.0f; F(K_DAL) = 0.0f;
+            }
+            if (LEARNED) seti(K_LV, 0u);
+            if (COUNT) path_iters = 1;
             if constexpr (SENSOR == kCamera) {
+                const uint32_t cell = geti(K_CELL);
+                const int px = (int)(cell % (uint32_t)P.width), py = (int)(cell / (uint32_t)P.width);
                 const float jx = 1.0f - u01(x.x), jy = 1.0f - u01(x.y);
                 const float sx = (2.0f * ((float)px + jx) * P.inv_width - 1.0f) * P.tan_half;
                 const float sy = (2.0f * ((float)py + jy) * P.inv_height - 1.0f) * P.tan_half * P.aspect;
@@ -339,9 +484,8 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
 #pragma unroll
                 for (int a = 0; a < 3; ++a) { vx[a] = q[a]; nd[a] = d[a]; }
                 kind = kMain;
-                c2 = 0u;
-                if (enters) { phase = PH_BEGIN; merge = true; mword = x.z; }
-                else evc = EV_ESCAPE;          // a path that misses the field scores 0
+                if (enters) { begin = true; tw = x.z; }
+                else phase = PH_END;           // a path that misses the field scores 0
             } else {
                 vx[0] = (1.0f - u01(x.x)) * S.Lper[0];
                 vx[1] = (1.0f - u01(x.y)) * S.Lper[1];
@@ -349,9 +493,8 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 if (!(vx[0] < S.Lper[0])) vx[0] = 0.0f;
                 if (!(vx[1] < S.Lper[1])) vx[1] = 0.0f;
                 kind = kSunDirect;
-                c2 = 3u;
-                Ts = 1.0f;
-                phase = PH_BEGIN;      // (its four words used up: the ray starts next time)
+                phase = PH_BEGIN;      // (its four words used up: the ray starts in the next pass)
+                F(K_TDIR) = 0.0f;
                 if constexpr (TERRAIN) {
                     // the surface point above (x, y), lifted along its normal;
                     // directions cosine-weighted about the normal; the direct
@@ -368,27 +511,32 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                         if (!(vx[a] >= 0.0f && vx[a] < S.Lper[a])) vx[a] = 0.0f;
                     }
                     cosine_about(n, u01(x.z), u01(x.w), nd);
-                    fz = n[2];
+                    F(K_FZ) = n[2];
                     const float ns = n[0] * S.sun[0] + n[1] * S.sun[1] + n[2] * S.sun[2];
-                    tdir = __fdividef(fmaxf(ns, 0.0f), n[2] * S.sun[2]);
-                    if (!(ns > 0.0f)) { kind = kMain; c2 = 0u; }     // self-shadowed: no direct sun ray
+                    F(K_TDIR) = __fdividef(fmaxf(ns, 0.0f), n[2] * S.sun[2]);
+                    if (!(ns > 0.0f)) kind = kMain;      // self-shadowed: no direct sun ray
                 } else {
                     cosine_up(u01(x.z), u01(x.w), nd);
                 }
             }
+            F(K_VX) = vx[0]; F(K_VY) = vx[1]; F(K_VZ) = vx[2];
+            F(K_NX) = nd[0]; F(K_NY) = nd[1]; F(K_NZ) = nd[2];
+            Ts = 1.0f;
         }
         mark(2);
-        if (ph == PH_VERTEX) {
+        if (vert) {
             // weight, estimate factor toward the sun, new direction, roulette
             const float xi1 = u01(x.x), xi2 = u01(x.y), xr = u01(x.z);
             const int order = (int)ev + 1;
             const bool score_it = (P.max_order == 0) || (order <= P.max_order);
-            if (!vground) {
+            float w = F(K_W), cf;
+            if (phase == PH_VERTEX) {
+                const float vk = F(K_VK);
                 const float om = omega_at(S, vk);
                 const float mu = R.d[0] * S.sun[0] + R.d[1] * S.sun[1] + R.d[2] * S.sun[2];
                 float ph = hg_pdf(S.g, mu);
                 float mu_new;
-                if (EXTRA && S.rayleigh) {
+                if (DECOMP && S.rayleigh) {
                     // Rayleigh clear air: the mixture phase function in the estimate;
                     // the species sampled with word 0 of the flight's vertex block
                     const float pc = cloud_scatter_share(S, vk);
@@ -401,11 +549,11 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 cf = score_it ? w * om * ph : 0.0f;
                 w *= om;
                 rotate_dir(R.d, mu_new, xi2, nd);
-                if (BATCH) {
-                    cfs = hg_dlog_dg(S.g, mu);
-                    sv_pending = hg_dlog_dg(S.g, mu_new);
+                if constexpr (BATCH) {
+                    F(K_CFS) = hg_dlog_dg(S.g, mu);
+                    F(K_SVP) = hg_dlog_dg(S.g, mu_new);
                     // d ln omega / d alpha = -k_cloud / (k omega) at this vertex
-                    if (EXTRA && om > 0.0f) sa -= __fdividef(fmaxf(vk - S.k_gas - S.k_clear, 0.0f), vk * om);
+                    if (EXTRA && om > 0.0f) F(K_SA) -= __fdividef(fmaxf(vk - S.k_gas - S.k_clear, 0.0f), vk * om);
                 }
                 if (COUNT) cnt[C_REAL]++;
             } else if constexpr (TERRAIN) {
@@ -421,6 +569,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                     if (!(vx[a] < S.Lper[a])) vx[a] -= S.Lper[a];
                     if (!(vx[a] >= 0.0f && vx[a] < S.Lper[a])) vx[a] = 0.0f;
                 }
+                F(K_VX) = vx[0]; F(K_VY) = vx[1]; F(K_VZ) = vx[2];
                 const float ns = n[0] * S.sun[0] + n[1] * S.sun[1] + n[2] * S.sun[2];
                 cf = (score_it && ns > 0.0f) ? w * (S.albedo * (1.0f / kPi)) * ns : 0.0f;
                 w *= S.albedo;
@@ -430,418 +579,330 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 cf = score_it ? w * (S.albedo * (1.0f / kPi)) * fmaxf(S.sun[2], 0.0f) : 0.0f;
                 w *= S.albedo;
                 cosine_up(xi1, xi2, nd);
-                if (BATCH) { cfs = 0.0f; sv_pending = 0.0f; }
+                if constexpr (BATCH) { F(K_CFS) = 0.0f; F(K_SVP) = 0.0f; }
                 if (COUNT) cnt[C_GROUND]++;
             }
-            term_after = (P.max_order > 0) && (order >= P.max_order);
+            bool term_after = (P.max_order > 0) && (order >= P.max_order);
             if (!term_after && w < 0.01f) {
                 if (xr * 0.01f <= w) w = 0.01f;
                 else term_after = true;
             }
+            if (term_after) seti(K_EV, ev | kTermAfter);
+            F(K_W) = w;
+            F(K_CF) = cf;
+            F(K_NX) = nd[0]; F(K_NY) = nd[1]; F(K_NZ) = nd[2];
             // (a ground facet turned away from the sun sends no sun ray)
-            if (score_it && (!TERRAIN || !vground || cf > 0.0f)) {
-                kind = kSunLocal;
-                c2 = (ev << 2) | 1u;
+            kind = kSunLocal;
+            if (score_it && (!TERRAIN || phase == PH_VERTEX || cf > 0.0f)) {
                 Ts = 1.0f;
-                phase = PH_BEGIN;
-                merge = true;
-                mword = x.w;     // word 3 of the vertex block
+                begin = true;
+                tw = x.w;        // word 3 of the vertex block
             } else {
                 Ts = 0.0f;
-                evc = EV_SUN_END;
+                phase = PH_SUN_END;
             }
         }
 
-        if (LEARNED && ph == PH_RESUME) {
-            // resume a path stopped at a learned vertex: state, network output,
-            // one-sample MIS direction, weight p_HG / q
-            const uint32_t slot = (uint32_t)pid;
-            const uint4 q0 = P.qin[4 * (size_t)slot], q1 = P.qin[4 * (size_t)slot + 1];
-            const uint4 q2 = P.qin[4 * (size_t)slot + 2], q3 = P.qin[4 * (size_t)slot + 3];
-            pid = (unsigned long long)q0.x | ((unsigned long long)q0.y << 32);
-            pend = pid + 1;
-            ev = q0.z;
-            lv = q0.w;
-            vx[0] = __uint_as_float(q1.x); vx[1] = __uint_as_float(q1.y); vx[2] = __uint_as_float(q1.z);
-            vk = __uint_as_float(q1.w);
-            R.d[0] = __uint_as_float(q2.x); R.d[1] = __uint_as_float(q2.y); R.d[2] = __uint_as_float(q2.z);
-            w = __uint_as_float(q2.w);
-            score = __uint_as_float(q3.x);
-            tdir = __uint_as_float(q3.y);
-            term_after = false;
-            if constexpr (SENSOR == kCamera) cell = (unsigned)(pid / P.spp);
-            kind = kMain;
-            c2 = ev << 2;
-            const uint4 xv = draw_block(pid, ev << 2, kBlockVertex, P.key);
-            const uint4 xl = draw_block(pid, ev << 2, kBlockVertex - 1u, P.key);
-            const float xi1 = u01(xv.x), xi2 = u01(xv.y), xr = u01(xv.z), xc = u01(xv.w), xlobe = u01(xl.x);
-            const int order = (int)ev + 1;
-            const bool score_it = (P.max_order == 0) || (order <= P.max_order);
-            const float om = omega_at(S, vk);
-            const float mu_s = R.d[0] * S.sun[0] + R.d[1] * S.sun[1] + R.d[2] * S.sun[2];
-            cf = score_it ? w * om * hg_pdf(S.g, mu_s) : 0.0f;
-            const float* mix = P.qin_mix + 48 * (size_t)slot;
-            if (xc <= P.mis_alpha) {
-                rotate_dir(R.d, hg_sample_mu(S.g, xi1), xi2, nd);
-            } else {
-                int j = 7;
+        if constexpr (LEARNED) {
+            if (phase == PH_RESUME) {
+                // resume a path stopped at a learned vertex: state, network output,
+                // one-sample MIS direction, weight p_HG / q
+                const uint32_t slot = (uint32_t)pid;
+                const uint4 q0 = P.qin[4 * (size_t)slot], q1 = P.qin[4 * (size_t)slot + 1];
+                const uint4 q2 = P.qin[4 * (size_t)slot + 2], q3 = P.qin[4 * (size_t)slot + 3];
+                const unsigned long long rpid = (unsigned long long)q0.x | ((unsigned long long)q0.y << 32);
+                set_pid(rpid);
+                const uint32_t rev = q0.z;
+                vx[0] = __uint_as_float(q1.x); vx[1] = __uint_as_float(q1.y); vx[2] = __uint_as_float(q1.z);
+                const float vk = __uint_as_float(q1.w);
+                float rd[3] = {__uint_as_float(q2.x), __uint_as_float(q2.y), __uint_as_float(q2.z)};
+                float w = __uint_as_float(q2.w);
+                const float score = __uint_as_float(q3.x);
+                F(K_SCORE) = score;
+                if (SENSOR == kFlux) F(K_TDIR) = __uint_as_float(q3.y);
+                if (SENSOR == kCamera) seti(K_CELL, (uint32_t)(rpid / P.spp));
+                const uint4 xv = draw_block(rpid, rev << 2, kBlockVertex, P.key);
+                const uint4 xl = draw_block(rpid, rev << 2, kBlockVertex - 1u, P.key);
+                const float xi1 = u01(xv.x), xi2 = u01(xv.y), xr = u01(xv.z), xc = u01(xv.w), xlobe = u01(xl.x);
+                const int order = (int)rev + 1;
+                const bool score_it = (P.max_order == 0) || (order <= P.max_order);
+                const float om = omega_at(S, vk);
+                const float mu_s = rd[0] * S.sun[0] + rd[1] * S.sun[1] + rd[2] * S.sun[2];
+                F(K_CF) = score_it ? w * om * hg_pdf(S.g, mu_s) : 0.0f;
+                const float* mix = P.qin_mix + 48 * (size_t)slot;
+                if (xc <= P.mis_alpha) {
+                    rotate_dir(rd, hg_sample_mu(S.g, xi1), xi2, nd);
+                } else {
+                    int j = 7;
 #pragma unroll
-                for (int i = 0; i < 7; ++i)
-                    if (j == 7 && xlobe <= __ldg(mix + 6 * i + 4)) j = i;
-                const float mu_l[3] = {__ldg(mix + 6 * j), __ldg(mix + 6 * j + 1), __ldg(mix + 6 * j + 2)};
-                const float kap = __ldg(mix + 6 * j + 3);
-                float cw = 1.0f + __logf(xi1 + (1.0f - xi1) * __expf(-2.0f * kap)) / kap;
-                cw = fminf(fmaxf(cw, -1.0f), 1.0f);
-                rotate_dir(mu_l, cw, xi2, nd);
-            }
-            const float phg = hg_pdf(S.g, R.d[0] * nd[0] + R.d[1] * nd[1] + R.d[2] * nd[2]);
-            // mixture density: sum of pi_j C(kappa_j) exp(kappa_j (mu_j . w - 1))
-            float qv = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float c = __ldg(mix + 6 * i) * nd[0] + __ldg(mix + 6 * i + 1) * nd[1] + __ldg(mix + 6 * i + 2) * nd[2];
-                qv += __ldg(mix + 6 * i + 5) * __expf(__ldg(mix + 6 * i + 3) * (c - 1.0f));
-            }
-            const float qmix = P.mis_alpha * phg + (1.0f - P.mis_alpha) * qv;
-            // training record: features, direction, score so far, w * omega
-            if (P.rec_count && slot < P.rec_slots) {
-                const unsigned idx = atomicAdd(P.rec_count, 1u);
-                if (idx < P.rec_cap) {
-                    P.rec_feat[2 * (size_t)idx] = P.qin_feat[2 * (size_t)slot];
-                    P.rec_feat[2 * (size_t)idx + 1] = P.qin_feat[2 * (size_t)slot + 1];
-                    P.rec_dir[3 * (size_t)idx] = nd[0];
-                    P.rec_dir[3 * (size_t)idx + 1] = nd[1];
-                    P.rec_dir[3 * (size_t)idx + 2] = nd[2];
-                    P.rec_val[4 * (size_t)idx] = score;
-                    P.rec_val[4 * (size_t)idx + 1] = w * om;
-                    P.rec_val[4 * (size_t)idx + 2] = 0.0f;
-                    P.rec_val[4 * (size_t)idx + 3] = __uint_as_float((uint32_t)(pid - P.path_base));
-                    cur_rec = idx;
+                    for (int i = 0; i < 7; ++i)
+                        if (j == 7 && xlobe <= __ldg(mix + 6 * i + 4)) j = i;
+                    const float mu_l[3] = {__ldg(mix + 6 * j), __ldg(mix + 6 * j + 1), __ldg(mix + 6 * j + 2)};
+                    const float kap = __ldg(mix + 6 * j + 3);
+                    float cw = 1.0f + __logf(xi1 + (1.0f - xi1) * __expf(-2.0f * kap)) / kap;
+                    cw = fminf(fmaxf(cw, -1.0f), 1.0f);
+                    rotate_dir(mu_l, cw, xi2, nd);
                 }
-            }
-            w *= om * __fdividef(phg, fmaxf(qmix, 1e-30f));
-            ++lv;
-            if (COUNT) cnt[C_REAL]++;
-            term_after = (P.max_order > 0) && (order >= P.max_order);
-            if (!term_after && w < 0.01f) {
-                if (xr * 0.01f <= w) w = 0.01f;
-                else term_after = true;
-            }
-            if (score_it) {
+                const float phg = hg_pdf(S.g, rd[0] * nd[0] + rd[1] * nd[1] + rd[2] * nd[2]);
+                // mixture density: sum of pi_j C(kappa_j) exp(kappa_j (mu_j . w - 1))
+                float qv = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float c = __ldg(mix + 6 * i) * nd[0] + __ldg(mix + 6 * i + 1) * nd[1] + __ldg(mix + 6 * i + 2) * nd[2];
+                    qv += __ldg(mix + 6 * i + 5) * __expf(__ldg(mix + 6 * i + 3) * (c - 1.0f));
+                }
+                const float qmix = P.mis_alpha * phg + (1.0f - P.mis_alpha) * qv;
+                // training record: features, direction, score so far, w * omega
+                if (P.rec_count && slot < P.rec_slots) {
+                    const unsigned idx = atomicAdd(P.rec_count, 1u);
+                    if (idx < P.rec_cap) {
+                        P.rec_feat[2 * (size_t)idx] = P.qin_feat[2 * (size_t)slot];
+                        P.rec_feat[2 * (size_t)idx + 1] = P.qin_feat[2 * (size_t)slot + 1];
+                        P.rec_dir[3 * (size_t)idx] = nd[0];
+                        P.rec_dir[3 * (size_t)idx + 1] = nd[1];
+                        P.rec_dir[3 * (size_t)idx + 2] = nd[2];
+                        P.rec_val[4 * (size_t)idx] = score;
+                        P.rec_val[4 * (size_t)idx + 1] = w * om;
+                        P.rec_val[4 * (size_t)idx + 2] = 0.0f;
+                        P.rec_val[4 * (size_t)idx + 3] = __uint_as_float((uint32_t)(rpid - P.path_base));
+                        seti(K_REC, idx);
+                    }
+                }
+                w *= om * __fdividef(phg, fmaxf(qmix, 1e-30f));
+                seti(K_LV, q0.w + 1u);
+                if (COUNT) cnt[C_REAL]++;
+                bool term_after = (P.max_order > 0) && (order >= P.max_order);
+                if (!term_after && w < 0.01f) {
+                    if (xr * 0.01f <= w) w = 0.01f;
+                    else term_after = true;
+                }
+                seti(K_EV, term_after ? rev | kTermAfter : rev);
+                F(K_W) = w;
+                F(K_VX) = vx[0]; F(K_VY) = vx[1]; F(K_VZ) = vx[2];
+                F(K_NX) = nd[0]; F(K_NY) = nd[1]; F(K_NZ) = nd[2];
                 kind = kSunLocal;
-                c2 = (ev << 2) | 1u;
-                Ts = 1.0f;
-                phase = PH_BEGIN;
-                merge = true;
-                mword = xl.y;    // word 1 of the lobe block
-            } else {
-                Ts = 0.0f;
-                evc = EV_SUN_END;
+                if (score_it) {
+                    Ts = 1.0f;
+                    begin = true;
+                    tw = xl.y;       // word 1 of the lobe block
+                } else {
+                    Ts = 0.0f;
+                    phase = PH_SUN_END;
+                }
             }
         }
         mark(5);
-        // a lane whose camera path start, vertex or resumed vertex set up a
-        // ray starts it now, so it skips one rare iteration and its wait;
-        // the ray's first optical depth comes from a word of the block that
-        // set it up (a flux path start uses all four words of its block, so
-        // its direct sun ray starts in a later iteration, from its own block)
-        const uint32_t tw = merge ? mword : x.x;
-        if (ph == PH_BEGIN || merge) {
-            // start a ray: the flight from vx along nd, or the sun ray from vx
+        // ---- ray starts: a camera path start or a vertex goes on into the
+        //      ray it set up (its first optical depth a word of the block
+        //      already drawn); a flight that follows a sun ray, and a flux
+        //      path's direct sun ray, draw their own block ---------------------
+        if (begin) {
+            // the flight from vx along nd, or the sun ray from vx
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const float d = (kind == kMain) ? nd[a] : S.sun[a];
                 R.o[a] = vx[a];
                 R.d[a] = d;
-                R.inv_d[a] = (d != 0.0f) ? __frcp_rn(d) : 0.0f;
                 R.v[a] = locate(vx[a], d, S.h[a], S.inv_h[a], 0, S.n[a] - 1);
             }
+            const uint2 e = __ldg(leaf_entry(S, R.v));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) R.inv_d[a] = (kind == kMain) ? dir_rcp(nd[a]) : S.inv_sun[a];
             R.t = 0.0f;
             R.steps = 0;
-            ptr = leaf_entry(S, R.v);
-            setup = true;
             tau = -__logf(u01(tw));
             blk = 1;
+            phase = PH_STEP;
             if constexpr (TERRAIN) {
                 // a sun ray that meets the surface is shadowed (found now: sun rays
                 // only start inside the relief layer at the ground or below hmax);
                 // a flight ends at the surface, found now when it starts inside the
                 // relief layer, else once its traversal reaches z = hmax
-                tg = __int_as_float(0x7f800000);
-                tpend = __int_as_float(0x7f800000);
+                tg = kInf;
+                tpend = kInf;
                 if (kind == kMain && R.o[2] > S.hmax) {
                     if (R.d[2] < 0.0f) tpend = __fdiv_rn(S.hmax - R.o[2], R.d[2]);
                 } else {
                     walk = true;
                 }
             }
+            finish_leaf<BF16>(S, R, e);
             if (COUNT) {
                 if (kind == kMain) cnt[C_FLIGHTS]++;
                 else cnt[C_SUN_RAYS]++;
             }
         }
-        if (TERRAIN && ph == PH_TERRAIN) {
-            walk = true;
-            tpend = __int_as_float(0x7f800000);
-            phase = PH_STEP;
-        }
-        if (TERRAIN && walk) {
-            const float th = terrain_hit(S, R.o, R.d);
-            if (kind == kMain) {
-                tg = th;
-            } else if (th < __int_as_float(0x7f800000)) {
-                Ts = 0.0f;
-                evc = EV_SUN_END;
-                ptr = nullptr;
-                setup = false;
+        if constexpr (TERRAIN) {
+            if (phase == PH_TERRAIN) {
+                walk = true;
+                tpend = kInf;
+                phase = PH_STEP;
+            }
+            if (walk) {
+                const float th = terrain_hit(S, R.o, R.d);
+                if (kind == kMain) {
+                    tg = th;
+                } else if (th < kInf) {
+                    Ts = 0.0f;
+                    phase = PH_SUN_END;
+                }
             }
         }
+        __syncwarp();
         mark(3);
-        if (ph == PH_STEP) {
-            // one step: to the tentative collision inside the leaf, or across
-            // the leaf's exit face; both share the point and voxel arithmetic
-            const bool at_ground = TERRAIN && !tent && tg <= R.texit;   // the surface cuts this leaf
-            const float tn = tent ? fminf(R.t + __fdividef(tau, Mt), TERRAIN ? fminf(R.texit, tg) : R.texit)
-                                  : (at_ground ? tg : R.texit);
-            if (decomp) Ts *= __expf(-R.mn * (tn - R.t));   // the control over this piece of the leaf
-            advance(S, R, tn, !tent && !at_ground, p, nv);
-            if (at_ground) {
-                // ground vertex at the surface hit (x, y wrapped into the domain)
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    if (p[a] < 0.0f) p[a] += S.Lper[a];
-                    if (!(p[a] < S.Lper[a])) p[a] -= S.Lper[a];
-                    if (!(p[a] >= 0.0f && p[a] < S.Lper[a])) p[a] = 0.0f;
+
+        // ==== steps: until enough lanes wait for a rare pass ====================
+        unsigned stepping;
+        do {
+            // (heightfield: a flight whose current leaf reaches down into the relief
+            //  layer first finds its ground hit, in a rare pass)
+            if (TERRAIN && phase == PH_STEP && R.texit >= tpend) phase = PH_TERRAIN;
+            if (COUNT) {
+                const unsigned st = __ballot_sync(kFull, phase == PH_STEP), lv = __ballot_sync(kFull, phase != PH_IDLE);
+                occ[0] += 1; occ[1] += __popc(lv); occ[2] += __popc(st); occ[5] += __popc(lv) - __popc(st);
+                occ[7] += 32 - __popc(lv);
+                if (phase == PH_STEP) ++path_iters;
+            }
+            if (phase == PH_STEP) {
+                // one step: to the tentative collision inside the leaf, or across
+                // the leaf's exit face; both share the point and voxel arithmetic.
+                // Tracking majorant: the leaf's M, or M - m for a sun ray in
+                // decomposition tracking (the minorant m is applied exactly)
+                const bool decomp = DECOMP && kind != kMain && P.sun_mode == MCRT_SUN_DECOMP;
+                const float Mt = decomp ? R.M - R.mn : R.M;
+                const float te = TERRAIN ? fminf(R.texit, tg) : R.texit;
+                const float Mseg = Mt * (te - R.t);
+                const bool tent = Mt > 0.0f && tau < Mseg;
+                const bool at_ground = TERRAIN && !tent && tg <= R.texit;   // the surface cuts this leaf
+                const float tn = tent ? fminf(R.t + __fdividef(tau, Mt), te) : (at_ground ? tg : R.texit);
+                if (decomp) Ts *= __expf(-R.mn * (tn - R.t));   // the control over this piece of the leaf
+                float p[3];
+                int nv[3];
+                advance(S, R, tn, !tent && !at_ground, p, nv);
+                const bool face = !tent && !at_ground;
+                int st = kInside;
+                uint2 e = make_uint2(0u, 0u);
+                if (face) {
+                    tau -= Mseg;
+                    float wdt;
+                    st = cross_face(S, R, p, nv, &wdt);
+                    if (TERRAIN) { tg -= wdt; tpend -= wdt; }   // a periodic wrap restarts the segment
+                    if (st == kInside) e = __ldg(leaf_entry(S, R.v));
                 }
-                vx[0] = p[0]; vx[1] = p[1]; vx[2] = fmaxf(p[2], 0.0f);
-                vground = true;
-                phase = PH_VERTEX;
-            } else if (tent) {
-                R.t = tn;
-                // a voxel leaf's majorant is the voxel itself: its tentative
-                // collision needs no load (k = M, so it is real; a sun ray's
-                // ratio 1 - k/M is 0)
-                if (R.lev != 0) {
-                    const size_t idx = brick_index(S, nv[0], nv[1], nv[2]);
-                    if (BF16) { ptr = reinterpret_cast<const uint2*>(S.vox16) + (idx >> 2); sub = (uint32_t)idx & 3u; }
-                    else { ptr = reinterpret_cast<const uint2*>(S.vox) + (idx >> 1); sub = (uint32_t)idx & 1u; }
-                }
-            } else {
-                tau -= Mseg;
-                float wdt;
-                st = cross_face(S, R, p, nv, &wdt);
-                if (TERRAIN) { tg -= wdt; tpend -= wdt; }   // a periodic wrap restarts the segment
-                if (st == kInside && decomp && Ts < 0.1f) {
-                    // roulette at a leaf crossing: word 3 of the next block, which it uses up
-                    if (u01(x.w) * 0.1f <= Ts) Ts = 0.1f;
-                    else { Ts = 0.0f; evc = EV_SUN_END; }
-                    ++blk;
-                }
-                if (st == kInside && evc == EV_NONE) {
-                    ptr = leaf_entry(S, R.v);
-                    setup = true;
+                // the block of a tentative collision, or of the roulette at a leaf
+                // crossing of decomposition tracking (word 3, which uses it up)
+                float k = R.M;
+                float ratio = 0.0f;
+                const bool roulette = DECOMP && decomp && face && st == kInside && Ts < 0.1f;
+                bool need = roulette;
+                if (COUNT && tent) ++tents;
+                if (tent) {
                     if (COUNT) {
-                        if (kind == kMain) cnt[C_LEAF]++;
-                        else cnt[C_SUN_LEAF]++;
+                        if (kind == kMain) cnt[C_TENT]++;
+                        else cnt[C_SUN_TENT]++;
                     }
-                } else if (st == kTop) {
-                    evc = (kind == kMain) ? EV_ESCAPE : EV_SUN_END;
-                } else {
+                    R.t = tn;
+                    if (R.msk != 0) {
+                        // (a voxel leaf's majorant is the voxel itself: no load)
+                        const size_t idx = brick_index(S, nv[0], nv[1], nv[2]);
+                        k = BF16 ? __uint_as_float((uint32_t)__ldg(S.vox16 + idx) << 16) : __ldg(S.vox + idx);
+                        k = __fadd_rn(k, S.k_gas);
+                        need = true;
+                    }
+                    if (kind != kMain && P.sun_mode != MCRT_SUN_DELTA) {
+                        if (decomp) ratio = 1.0f - __fdividef(k - R.mn, R.M - R.mn);
+                        else ratio = 1.0f - __fdividef(k, R.M);
+                        // (0 in a voxel leaf but for rounding)
+                        need = need || ratio > 0.0f;
+                    }
+                }
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                if (need) {
+                    const uint32_t ev = geti(K_EV) & ~kTermAfter;
+                    x = draw_block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk,
+                                   BATCH ? P.items[geti(K_CELL)].key : P.key);
+                }
+                if (tent) {
+                    if (need) ++blk;
+                    const float u0 = u01(x.x);
                     if (kind == kMain) {
-                        // ground hit: the vertex is handled in a later iteration
-                        p[2] = 0.0f;
-                        p[0] = fminf(fmaxf(p[0], 0.0f), S.Lper[0]);
-                        p[1] = fminf(fmaxf(p[1], 0.0f), S.Lper[1]);
-                        if (!(p[0] < S.Lper[0])) p[0] = 0.0f;
-                        if (!(p[1] < S.Lper[1])) p[1] = 0.0f;
-                        vx[0] = p[0]; vx[1] = p[1]; vx[2] = p[2];
-                        vground = true;
-                        phase = PH_VERTEX;
+                        if (u0 * R.M <= k) {
+                            F(K_VX) = p[0]; F(K_VY) = p[1]; F(K_VZ) = p[2];
+                            F(K_VK) = k;
+                            phase = PH_VERTEX;
+                            if constexpr (LEARNED) {
+                                if (geti(K_LV) < (uint32_t)P.n_learned) {
+                                    phase = PH_SUSPEND;
+                                    R.v[0] = nv[0]; R.v[1] = nv[1]; R.v[2] = nv[2];
+                                }
+                            }
+                        }
+                    } else if (P.sun_mode == MCRT_SUN_DELTA) {
+                        if (u0 * R.M <= k) { Ts = 0.0f; phase = PH_SUN_END; }
                     } else {
-                        Ts = 0.0f;
-                        evc = EV_SUN_END;
-                    }
-                }
-            }
-        }
-        mark(4);
-        // ---- the one load: voxel word or leaf-map entry ---------------------
-        uint2 val = make_uint2(0u, 0u);
-        if (ptr) val = __ldg(ptr);
-        if (COUNT) asm volatile("" ::"r"(val.x), "r"(val.y));   // charge the load latency here
-        mark(6);
-
-        // ---- after the load ----------------------------------------------------
-        if (setup) {
-            finish_leaf<BF16>(S, R, val);
-            if (ph == PH_BEGIN || merge) phase = PH_STEP;
-            else if (R.steps > P.max_steps) evc = EV_ABORT;
-        } else if (tent) {
-            float kv;
-            if (BF16) {
-                const uint32_t wd = (sub & 2u) ? val.y : val.x;
-                kv = __uint_as_float(((wd >> ((sub & 1u) * 16u)) & 0xFFFFu) << 16);
-            } else {
-                kv = __uint_as_float(sub ? val.y : val.x);
-            }
-            const float k = R.lev == 0 ? R.M : __fadd_rn(kv, S.k_gas);
-            ++blk;
-            const float u0 = u01(x.x);
-            const float nt = -__logf(u01(x.y));
-            if (kind == kMain) {
-                if (COUNT) cnt[C_TENT]++;
-                if (u0 * R.M <= k) {
-                    vx[0] = p[0]; vx[1] = p[1]; vx[2] = p[2];
-                    vk = k;
-                    vground = false;
-                    phase = PH_VERTEX;
-                    if (LEARNED && lv < (uint32_t)P.n_learned) suspend = true;
-                } else {
-                    tau = nt;
-                }
-            } else {
-                if (COUNT) cnt[C_SUN_TENT]++;
-                bool ended = false;
-                if (P.sun_mode == MCRT_SUN_DELTA) {
-                    if (u0 * R.M <= k) { Ts = 0.0f; ended = true; }
-                } else {
-                    if (EXTRA && P.sun_mode == MCRT_SUN_DECOMP) Ts *= 1.0f - __fdividef(k - R.mn, R.M - R.mn);
-                    else Ts *= 1.0f - __fdividef(k, R.M);
-                    if (!(Ts > 0.0f)) { Ts = 0.0f; ended = true; }
-                    else if (Ts < 0.1f) {
-                        if (u0 * 0.1f <= Ts) Ts = 0.1f;
-                        else { Ts = 0.0f; ended = true; }
-                    }
-                }
-                if (ended) evc = EV_SUN_END;
-                else tau = nt;
-            }
-        }
-
-        mark(7);
-        // ---- end of a ray or of the path -------------------------------------
-        if (evc != EV_NONE) {
-            bool path_done = false;
-            if (evc == EV_ABORT) {
-                if (COUNT) cnt[C_ABORT]++;
-                if (kind == kMain) path_done = true;
-                else { Ts = 0.0f; evc = EV_SUN_END; }
-            }
-            if (evc == EV_SUN_END) {
-                if (kind == kSunDirect) {
-                    tdir = TERRAIN ? tdir * Ts : Ts;
-                    ev = 0;
-                    kind = kMain;
-                    c2 = 0u;
-                    phase = PH_BEGIN;
-                } else {
-                    score += cf * Ts;
-                    if (BATCH) {
-                        dscore += cf * Ts * (sg + cfs);
-                        if (EXTRA) dal += cf * Ts * sa;
-                        sg += sv_pending;
-                    }
-                    if (LEARNED && cur_rec != 0xFFFFFFFFu) {
-                        P.rec_val[4 * (size_t)cur_rec + 2] = cf * Ts;
-                        cur_rec = 0xFFFFFFFFu;
-                    }
-                    if (term_after) {
-                        path_done = true;
-                    } else {
-                        ++ev;
-                        kind = kMain;
-                        c2 = ev << 2;
-                        phase = PH_BEGIN;
-                    }
-                }
-            }
-            if (evc == EV_ESCAPE) path_done = true;
-            if (path_done) {
-                if constexpr (SENSOR == kCamera) {
-                    acc[0] += score;
-                    acc[1] += score * score;
-                } else {
-                    const float pi_over_mu0 = __fdividef(kPi, TERRAIN ? fz * S.sun[2] : S.sun[2]);
-                    const float tf = pi_over_mu0 * score;
-                    const float tt = tdir + tf;
-                    acc[0] += tdir; acc[1] += tdir * tdir;
-                    acc[2] += tf; acc[3] += tf * tf;
-                    acc[4] += tt; acc[5] += tt * tt;
-                    if constexpr (BATCH) {
-                        const float dt = pi_over_mu0 * dscore;
-                        acc[6] += dt; acc[7] += dt * dt;
-                        if (EXTRA) {
-                            const float da = pi_over_mu0 * dal;
-                            acc[8] += da; acc[9] += da * da;
+                        Ts *= ratio;
+                        if (!(Ts > 0.0f)) { Ts = 0.0f; phase = PH_SUN_END; }
+                        else if (Ts < 0.1f) {
+                            if (u0 * 0.1f <= Ts) Ts = 0.1f;
+                            else { Ts = 0.0f; phase = PH_SUN_END; }
                         }
                     }
-                }
-                if (COUNT) {
-                    cnt[C_PATHS]++;
-                    max_iters = max(max_iters, path_iters);
-                }
-                if (LEARNED && P.final_score) P.final_score[pid - P.path_base] = score;
-                ++pid;
-                phase = (pid < pend) ? PH_START : PH_IDLE;
-            }
-        }
-        // ---- stop paths at a learned vertex: state and features to the queue
-        if (LEARNED) {
-            const unsigned smask = __ballot_sync(kFull, suspend);
-            if (smask) {
-                const int leader = __ffs(smask) - 1;
-                unsigned base = 0;
-                if (lane == leader) base = atomicAdd(P.qout_count, (unsigned)__popc(smask));
-                base = __shfl_sync(kFull, base, leader);
-                if (suspend) {
-                    const unsigned slot = base + (unsigned)__popc(smask & lt_mask);
-                    if (slot < P.qout_cap) {
-                        // features: position in [-1, 1], incoming direction, ln(k), ln(M1), ln(M2)
-                        const float Lz = (float)S.n[2] * S.h[2];
-                        float f[9];
-                        f[0] = 2.0f * vx[0] / S.Lper[0] - 1.0f;
-                        f[1] = 2.0f * vx[1] / S.Lper[1] - 1.0f;
-                        f[2] = 2.0f * vx[2] / Lz - 1.0f;
-                        f[3] = R.d[0]; f[4] = R.d[1]; f[5] = R.d[2];
-                        f[6] = logf(vk + 1e-6f);
-                        const float M1 = __ldg(P.pyr1 + ((size_t)(nv[2] >> 3) * P.d1[1] + (nv[1] >> 3)) * P.d1[0] +
-                                               (nv[0] >> 3));
-                        const int s2 = 3 * P.lev2;
-                        const float M2 = __ldg(P.pyr2 + ((size_t)(nv[2] >> s2) * P.d2[1] + (nv[1] >> s2)) * P.d2[0] +
-                                               (nv[0] >> s2));
-                        f[7] = logf(M1 + S.k_gas + 1e-6f);
-                        f[8] = logf(M2 + S.k_gas + 1e-6f);
-                        uint32_t pk[8];
+                    if (phase == PH_STEP) tau = -__logf(u01(x.y));
+                } else if (at_ground) {
+                    // ground vertex at the surface hit (x, y wrapped into the domain)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const __nv_bfloat162 v = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-                            pk[i] = *reinterpret_cast<const uint32_t*>(&v);
-                        }
-                        pk[4] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(f[8]));
-                        pk[5] = pk[6] = pk[7] = 0u;
-                        P.qout_feat[2 * (size_t)slot] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        P.qout_feat[2 * (size_t)slot + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-                        P.qout[4 * (size_t)slot] = make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), ev, lv);
-                        P.qout[4 * (size_t)slot + 1] = make_uint4(__float_as_uint(vx[0]), __float_as_uint(vx[1]),
-                                                                  __float_as_uint(vx[2]), __float_as_uint(vk));
-                        P.qout[4 * (size_t)slot + 2] = make_uint4(__float_as_uint(R.d[0]), __float_as_uint(R.d[1]),
-                                                                  __float_as_uint(R.d[2]), __float_as_uint(w));
-                        P.qout[4 * (size_t)slot + 3] = make_uint4(__float_as_uint(score), __float_as_uint(tdir), 0u, 0u);
+                    for (int a = 0; a < 2; ++a) {
+                        if (p[a] < 0.0f) p[a] += S.Lper[a];
+                        if (!(p[a] < S.Lper[a])) p[a] -= S.Lper[a];
+                        if (!(p[a] >= 0.0f && p[a] < S.Lper[a])) p[a] = 0.0f;
                     }
-                    suspend = false;
-                    ++pid;
-                    phase = (pid < pend) ? PH_START : PH_IDLE;
+                    F(K_VX) = p[0]; F(K_VY) = p[1]; F(K_VZ) = fmaxf(p[2], 0.0f);
+                    phase = PH_GROUND;
+                } else if (st == kInside) {
+                    if (roulette) {
+                        ++blk;
+                        if (u01(x.w) * 0.1f <= Ts) Ts = 0.1f;
+                        else { Ts = 0.0f; phase = PH_SUN_END; }
+                    }
+                    if (!roulette || phase == PH_STEP) {
+                        if (COUNT) {
+                            if (kind == kMain) cnt[C_LEAF]++;
+                            else cnt[C_SUN_LEAF]++;
+                        }
+                        finish_leaf<BF16>(S, R, e);
+                        if (R.steps > P.max_steps) {
+                            if (COUNT) cnt[C_ABORT]++;
+                            Ts = 0.0f;
+                            phase = kind == kMain ? PH_END : PH_SUN_END;
+                        }
+                    }
+                } else if (kind != kMain) {
+                    if (st == kGround) Ts = 0.0f;
+                    phase = PH_SUN_END;
+                } else if (st == kTop) {
+                    phase = PH_END;
+                } else {
+                    // ground hit: the vertex is handled in the next rare pass
+                    p[0] = fminf(fmaxf(p[0], 0.0f), S.Lper[0]);
+                    p[1] = fminf(fmaxf(p[1], 0.0f), S.Lper[1]);
+                    if (!(p[0] < S.Lper[0])) p[0] = 0.0f;
+                    if (!(p[1] < S.Lper[1])) p[1] = 0.0f;
+                    F(K_VX) = p[0]; F(K_VY) = p[1]; F(K_VZ) = 0.0f;
+                    phase = PH_GROUND;
                 }
             }
-        }
-        mark(8);
+            stepping = __ballot_sync(kFull, phase == PH_STEP);
+            --budget;
+        } while ((__popc(stepping) >= P.min_steppers || stepping == live) && stepping != 0u && budget > 0);
+        mark(4);
     }
 
     // ---- partial sums left by a deadline / cancel exit ------------------------
-    if (chunk) {
+    if (phase != PH_IDLE && phase != PH_CLAIM) {
 #pragma unroll
         for (int q = 0; q < 2 * NQ; ++q)
-            if (acc[q] != 0.0f) atomicAdd(((q & 1) ? P.s2 : P.s1) + (size_t)cell * NQ + (q >> 1), (double)acc[q]);
+            if (F(K_ACC + q) != 0.0f)
+                atomicAdd(((q & 1) ? P.s2 : P.s1) + (size_t)geti(K_CELL) * NQ + (q >> 1), (double)F(K_ACC + q));
     }
     if (COUNT) {
 #pragma unroll
@@ -850,13 +911,17 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
             for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
             if (lane == 0 && a) atomicAdd(P.counters + q, a);
         }
+        unsigned long long nt = tents;
+        for (int o = 16; o > 0; o >>= 1) nt += __shfl_xor_sync(kFull, nt, o);
+        if (lane == 0) atomicAdd(P.counters + C_OCC + 3, nt);
         unsigned mi = max_iters;
         for (int o = 16; o > 0; o >>= 1) mi = max(mi, __shfl_xor_sync(kFull, mi, o));
         if (lane == 0) {
 #pragma unroll
             for (int q = 0; q < kSections; ++q) atomicAdd(P.counters + C_SEC + q, sec[q]);
 #pragma unroll
-            for (int q = 0; q < kOcc; ++q) atomicAdd(P.counters + C_OCC + q, occ[q]);
+            for (int q = 0; q < kOcc; ++q)
+                if (q != 3) atomicAdd(P.counters + C_OCC + q, occ[q]);
             const uint64_t t_end = globaltimer_ns();
             atomicMax(P.counters + C_MAX_ITERS, (unsigned long long)mi);
             if (t_dry) atomicMax(P.counters + C_T_DRY, (unsigned long long)(t_dry - t_start));
@@ -894,10 +959,11 @@ __global__ void debug_dda_kernel(DevScene S, float ox, float oy, float oz, float
     int n = 0, status = 0;
     for (;;) {
         if (n >= cap) { status = 3; break; }
-        cells[4 * n + 0] = R.lev / S.lb;      // level of the tracked grid
-        cells[4 * n + 1] = R.v[0] >> R.lev;
-        cells[4 * n + 2] = R.v[1] >> R.lev;
-        cells[4 * n + 3] = R.v[2] >> R.lev;
+        const int lev = __popc((unsigned)R.msk);
+        cells[4 * n + 0] = lev / S.lb;        // level of the tracked grid
+        cells[4 * n + 1] = R.v[0] >> lev;
+        cells[4 * n + 2] = R.v[1] >> lev;
+        cells[4 * n + 3] = R.v[2] >> lev;
         tio[2 * n + 0] = __fadd_rn(tbase, R.t);
         tio[2 * n + 1] = __fadd_rn(tbase, R.texit);
         ++n;

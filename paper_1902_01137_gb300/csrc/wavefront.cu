@@ -129,7 +129,7 @@ __device__ __forceinline__ void wf_ray_start(const DevScene& S, Ray& R, const fl
     for (int a = 0; a < 3; ++a) {
         R.o[a] = o[a];
         R.d[a] = d[a];
-        R.inv_d[a] = (d[a] != 0.0f) ? __frcp_rn(d[a]) : 0.0f;
+        R.inv_d[a] = dir_rcp(d[a]);
         R.v[a] = locate(o[a], d[a], S.h[a], S.inv_h[a], 0, S.n[a] - 1);
     }
     R.t = 0.0f;
@@ -181,7 +181,7 @@ __device__ __forceinline__ bool wf_step(const DevScene& S, Ray& R, float& tau, f
     advance(S, R, tn, !tent, p, nv);
     if (tent) {
         R.t = tn;
-        *k = R.lev == 0 ? R.M : __fadd_rn(kfetch<BF16>(S, nv[0], nv[1], nv[2]), S.k_gas);
+        *k = R.msk == 0 ? R.M : __fadd_rn(kfetch<BF16>(S, nv[0], nv[1], nv[2]), S.k_gas);
         return true;
     }
     tau -= Mseg;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kWfBlock) wf_flight_kernel(const __grid_consta
                 for (int a = 0; a < 3; ++a) {
                     R.o[a] = o[a];
                     R.d[a] = d[a];
-                    R.inv_d[a] = (d[a] != 0.0f) ? __frcp_rn(d[a]) : 0.0f;
+                    R.inv_d[a] = dir_rcp(d[a]);
                     R.v[a] = (int)F.vox[a][i];
                 }
                 R.t = F.t[i];
