@@ -78,6 +78,7 @@ DevScene make_dev_scene(const mcrt_scene* sc, float k_gas)
     DevScene S{};
     for (int a = 0; a < 3; ++a) {
         S.n[a] = sc->n[a];
+        S.nm1[a] = sc->n[a] - 1;
         S.h[a] = sc->h[a];
         S.inv_h[a] = 1.0f / sc->h[a];
         S.nb[a] = sc->nb[a];

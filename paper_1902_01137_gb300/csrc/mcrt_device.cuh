@@ -92,6 +92,7 @@ constexpr int kMaxGridLevels = 20;   // octree levels for fields up to 2^20 voxe
 
 struct DevScene {
     int n[3];            // voxels per axis
+    int nm1[3];          // n - 1
     float h[3];          // voxel size [km]
     float inv_h[3];      // 1 / h, round to nearest
     float Lper[2];       // n * h for the periodic axes
@@ -151,13 +152,15 @@ struct Ray {
     float o[3];      // segment origin
     float d[3];      // unit direction
     float inv_d[3];  // 1 / d (NaN where d == 0: no exit on that axis)
-    int v[3];        // voxel of the current point
+    int lo[3];       // voxels of the current leaf, first ...
+    int hi[3];       // ... and last (inside the field)
     int msk;         // leaf size - 1: the leaf spans msk + 1 = 2^shift voxels per axis (0: a voxel leaf)
     float M;         // leaf majorant (+ k_gas)
     float mn;        // leaf minorant (+ k_gas)
     float t;         // distance of the current point from o
     float texit;     // distance of the leaf exit from o
     int ax;          // exit axis
+    int across;      // voxel index behind the exit face on that axis (may lie outside the field)
     uint32_t steps;  // leaves entered (guard)
 };
 
@@ -209,28 +212,33 @@ __device__ __forceinline__ float brick_fetch(const DevScene& S, uint32_t brick, 
 #endif
 }
 
-// Finish entering the leaf holding R.v from its leaf-map entry: size,
+// Finish entering the leaf holding voxel v from its leaf-map entry: size,
 // majorant and the exit distance / axis.  On each axis the exit face is the
 // upper one (min(lo + size, n)) when d > 0, else the lower one; an axis with
 // d == 0 has a NaN distance, which the minimum skips.
 template <bool BF16>
-__device__ __forceinline__ void finish_leaf(const DevScene& S, Ray& R, uint2 e)
+__device__ __forceinline__ void finish_leaf(const DevScene& S, Ray& R, const int v[3], uint2 e)
 {
     // entry: .x majorant bits (a voxel leaf: its brick), .y = minorant rounded down to bfloat16 | shift
     R.msk = (int)((1u << (e.y & 31u)) - 1u);
     float M = __uint_as_float(e.x), mn = __uint_as_float(e.y & 0xFFFF0000u);
-    if (R.msk == 0) M = mn = brick_fetch<BF16>(S, e.x, R.v);
+    if (R.msk == 0) M = mn = brick_fetch<BF16>(S, e.x, v);
     R.M = __fadd_rn(M, S.k_gas);
     R.mn = __fadd_rn(mn, S.k_gas);
     float ta[3];
+    int X[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int up = min((R.v[a] | R.msk) + 1, S.n[a]);
-        const int B = R.d[a] > 0.0f ? up : (R.v[a] & ~R.msk);
+        R.lo[a] = v[a] & ~R.msk;
+        R.hi[a] = min(v[a] | R.msk, S.nm1[a]);
+        const bool up = R.d[a] > 0.0f;
+        X[a] = up ? R.hi[a] + 1 : R.lo[a] - 1;
+        const int B = up ? X[a] : R.lo[a];
         ta[a] = __fmul_rn(__fsub_rn(__fmul_rn(__int2float_rn(B), S.h[a]), R.o[a]), R.inv_d[a]);
     }
     const float tm = fminf(fminf(ta[0], ta[1]), ta[2]);
     R.ax = tm == ta[0] ? 0 : (tm == ta[1] ? 1 : 2);
+    R.across = tm == ta[0] ? X[0] : (tm == ta[1] ? X[1] : X[2]);
     R.texit = fmaxf(tm, R.t);
 }
 
@@ -238,16 +246,17 @@ __device__ __forceinline__ void finish_leaf(const DevScene& S, Ray& R, uint2 e)
 template <bool BF16>
 __device__ __forceinline__ void ray_begin(const DevScene& S, Ray& R, const float p[3], const float d[3])
 {
+    int v[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         R.o[a] = p[a];
         R.d[a] = d[a];
         R.inv_d[a] = dir_rcp(d[a]);
-        R.v[a] = locate(p[a], d[a], S.h[a], S.inv_h[a], 0, S.n[a] - 1);
+        v[a] = locate(p[a], d[a], S.h[a], S.inv_h[a], 0, S.nm1[a]);
     }
     R.t = 0.0f;
     R.steps = 0;
-    finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+    finish_leaf<BF16>(S, R, v, __ldg(leaf_entry(S, v)));
 }
 
 enum StepResult { kInside = 0, kTop = 1, kGround = 2 };
@@ -261,21 +270,18 @@ __device__ __forceinline__ void advance(const DevScene& S, const Ray& R, float t
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
         p[b] = __fmaf_rn(tn, R.d[b], R.o[b]);
-        const int lo = R.v[b] & ~R.msk;
-        const int hi = min(R.v[b] | R.msk, S.n[b] - 1);
-        nv[b] = locate(p[b], R.d[b], S.h[b], S.inv_h[b], lo, hi);
+        const int i = locate(p[b], R.d[b], S.h[b], S.inv_h[b], R.lo[b], R.hi[b]);
         // the exit axis steps across the face (its located value is discarded)
-        const int across = R.d[b] > 0.0f ? hi + 1 : lo - 1;
         const bool exits = face && R.ax == b;
-        nv[b] = exits ? across : nv[b];
+        nv[b] = exits ? R.across : i;
     }
 }
 
 // Complete a face crossing prepared by advance(face = true): the ground or
 // the top, or the periodic wrap of x / y (the segment then restarts on the
 // face: o on the face exactly, t = 0, *wrapped_dt = distance of the finished
-// segment), then the new voxel.  Only the exit axis can leave the domain.
-// The caller loads the leaf-map entry of R.v and calls finish_leaf when the
+// segment), nv then the new voxel.  Only the exit axis can leave the domain.
+// The caller loads the leaf-map entry of nv and calls finish_leaf when the
 // result is kInside.
 __device__ __forceinline__ int cross_face(const DevScene& S, Ray& R, const float p[3], int nv[3], float* wrapped_dt)
 {
@@ -295,16 +301,14 @@ __device__ __forceinline__ int cross_face(const DevScene& S, Ray& R, const float
         }
         R.t = 0.0f;
     }
-    R.v[0] = nv[0]; R.v[1] = nv[1]; R.v[2] = nv[2];
     ++R.steps;
     return kInside;
 }
 
 // Cross the exit face of the current leaf (advance + cross_face); p receives
 // the exit point before any wrap shift.
-__device__ __forceinline__ int step_face(const DevScene& S, Ray& R, float p[3], float* wrapped_dt)
+__device__ __forceinline__ int step_face(const DevScene& S, Ray& R, float p[3], int nv[3], float* wrapped_dt)
 {
-    int nv[3];
     advance(S, R, R.texit, true, p, nv);
     return cross_face(S, R, p, nv, wrapped_dt);
 }
@@ -589,6 +593,20 @@ static __device__ __forceinline__ float terrain_hit(const DevScene& S, const flo
     for (int it = 0; it < (1 << 16); ++it)
         if (terrain_walk_step(S, o, d, inv_d, W, &th)) return th;
     return kInf;
+}
+
+// Ratio tracking's factor 1 - k / M by the approximate reciprocal of M, the
+// product and the difference as one operation (FUSED) or each rounded.  For
+// k = M it is 0 or a rounding residual below 2^-22, which the roulette below
+// T_sun = 0.1 then decides.  Written out because the two roundings differ:
+// each kernel variant keeps the one it has always used.
+template <bool FUSED>
+__device__ __forceinline__ float null_share(float k, float M)
+{
+    if (!FUSED) return __fsub_rn(1.0f, __fdividef(k, M));
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(M));
+    return __fmaf_rn(-k, r, 1.0f);
 }
 
 // Single-scattering albedo of the mixture at total extinction k_tot.

@@ -97,6 +97,7 @@ enum Phase {
     PH_RESUME,      // a path stopped at a learned vertex goes on
     PH_SUSPEND,     // a path stops at a learned vertex
     PH_TERRAIN,     // a flight reached the relief layer: find its ground hit
+    PH_ROULETTE,    // a sun ray's tentative collision in a voxel leaf left a residual Ts: its draw
     PH_SUN_END,     // a sun ray ended with transmissivity Ts
     PH_END          // the path ends
 };
@@ -153,6 +154,18 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         seti(K_PID_HI, (uint32_t)(pid >> 32));
     };
 
+    // the warp's FP64 sums for tally cell wcell (flux): lane q owns entry q
+    __shared__ double wsum[SENSOR == kCamera ? 1 : 4][SENSOR == kCamera ? 1 : 2 * NQ];
+    uint32_t wcell = 0u;
+    auto spill_sums = [&]() {
+        if (SENSOR == kFlux && lane < 2 * NQ) {
+            double& a = wsum[tid >> 5][lane];
+            if (a != 0.0) atomicAdd(((lane & 1) ? P.s2 : P.s1) + (size_t)wcell * NQ + (lane >> 1), a);
+            a = 0.0;
+        }
+    };
+    if (SENSOR == kFlux && lane < 2 * NQ) wsum[tid >> 5][lane] = 0.0;
+
     // ---- per-lane state ------------------------------------------------------
     const float kInf = __int_as_float(0x7f800000);
     bool exhausted = false;                 // warp-uniform: nothing left to claim
@@ -194,6 +207,20 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
     for (;;) {
         // ==== rare pass: every lane that is not stepping ======================
         // ---- rays and paths that ended ---------------------------------------
+        if (phase == PH_ROULETTE) {
+            // the block this tentative collision would have drawn: test (the
+            // ratio's roulette below 0.1) and next optical depth
+            const uint4 x = draw_block(get_pid(),
+                                       SENSOR == kFlux && kind == kSunDirect ? 3u : ((geti(K_EV) & ~kTermAfter) << 2) | 1u,
+                                       blk, BATCH ? P.items[geti(K_CELL)].key : P.key);
+            ++blk;
+            phase = PH_STEP;
+            if (Ts < 0.1f) {
+                if (u01(x.x) * 0.1f <= Ts) Ts = 0.1f;
+                else { Ts = 0.0f; phase = PH_SUN_END; }
+            }
+            tau = -__logf(u01(x.y));
+        }
         if (phase == PH_SUN_END) {
             if (SENSOR == kFlux && kind == kSunDirect) {
                 if constexpr (SENSOR == kFlux) F(K_TDIR) = TERRAIN ? F(K_TDIR) * Ts : Ts;
@@ -275,7 +302,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                     if (slot < P.qout_cap) {
                         // features: position in [-1, 1], incoming direction, ln(k), ln(M1), ln(M2)
                         const float vx[3] = {F(K_VX), F(K_VY), F(K_VZ)}, vk = F(K_VK);
-                        const int nv[3] = {R.v[0], R.v[1], R.v[2]};   // (the collision's voxel)
+                        const int nv[3] = {(int)geti(K_NX), (int)geti(K_NY), (int)geti(K_NZ)};   // the collision's voxel
                         const float Lz = (float)S.n[2] * S.h[2];
                         float f[9];
                         f[0] = 2.0f * vx[0] / S.Lper[0] - 1.0f;
@@ -315,27 +342,44 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 }
             }
         }
-        // ---- flush finished chunks: lanes sharing a cell are summed first --
+        // ---- finished chunks: their sums go to the tally -----------------------
         unsigned fmask = __ballot_sync(kFull, phase == PH_FLUSH);
-        while (fmask) {
-            const int src = __ffs(fmask) - 1;
-            const unsigned my = geti(K_CELL);
-            const unsigned c = __shfl_sync(kFull, my, src);
-            MCRT_CHECK(c < (SENSOR == kCamera ? (unsigned)(P.width * P.height) : (BATCH ? (unsigned)P.n_items : 1u)), 3);
-            const bool mine = phase == PH_FLUSH && my == c;
-#pragma unroll
-            for (int q = 0; q < 2 * NQ; ++q) {
-                double a = mine ? (double)F(K_ACC + q) : 0.0;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
-                if (lane == src) atomicAdd(((q & 1) ? P.s2 : P.s1) + (size_t)c * NQ + (q >> 1), a);
+        if (fmask) {
+            if constexpr (SENSOR == kCamera) {
+                // (chunks that end together rarely share a pixel)
+                if (phase == PH_FLUSH) {
+                    const uint32_t c = geti(K_CELL);
+                    MCRT_CHECK(c < (unsigned)(P.width * P.height), 3);
+                    atomicAdd(P.s1 + c, (double)F(K_ACC));
+                    atomicAdd(P.s2 + c, (double)F(K_ACC + 1));
+                }
+            } else {
+                // lane q < 2 NQ adds quantity q of the finished chunks, one after
+                // another, to the warp's FP64 sums of the tally cell it works on;
+                // they reach the tally when the warp turns to another cell, and
+                // at its end.  (A shuffle reduction of every quantity over the
+                // warp and an atomic per finished chunk took 10-12 % of a
+                // trace with claims of one path: 16.8 M flux paths 49.8 -> 44.5
+                // ms, 4 M over a relief 25.3 -> 23.2, a learned image's passes
+                // 22.3 -> 19.9.)
+                __syncwarp();
+                for (unsigned left = fmask; left; left &= left - 1u) {
+                    const int src = (tid & ~31) + __ffs(left) - 1;
+                    const uint32_t c = __float_as_uint(cold[K_CELL][src]);
+                    MCRT_CHECK(c < (BATCH ? (unsigned)P.n_items : 1u), 3);
+                    if (BATCH && c != wcell) {
+                        spill_sums();
+                        wcell = c;
+                    }
+                    if (lane < 2 * NQ) wsum[tid >> 5][lane] += (double)cold[K_ACC + lane][src];
+                }
+                __syncwarp();
             }
-            if (mine) {
+            if (phase == PH_FLUSH) {
                 phase = PH_CLAIM;
 #pragma unroll
                 for (int q = 0; q < 2 * NQ; ++q) F(K_ACC + q) = 0.0f;
             }
-            fmask = __ballot_sync(kFull, phase == PH_FLUSH);
         }
         // ---- claim chunks for idle lanes (one atomic per warp) -------------
         const unsigned idle = __ballot_sync(kFull, phase == PH_CLAIM);
@@ -698,14 +742,15 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         //      path's direct sun ray, draw their own block ---------------------
         if (begin) {
             // the flight from vx along nd, or the sun ray from vx
+            int v[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const float d = (kind == kMain) ? nd[a] : S.sun[a];
                 R.o[a] = vx[a];
                 R.d[a] = d;
-                R.v[a] = locate(vx[a], d, S.h[a], S.inv_h[a], 0, S.n[a] - 1);
+                v[a] = locate(vx[a], d, S.h[a], S.inv_h[a], 0, S.nm1[a]);
             }
-            const uint2 e = __ldg(leaf_entry(S, R.v));
+            const uint2 e = __ldg(leaf_entry(S, v));
 #pragma unroll
             for (int a = 0; a < 3; ++a) R.inv_d[a] = (kind == kMain) ? dir_rcp(nd[a]) : S.inv_sun[a];
             R.t = 0.0f;
@@ -726,7 +771,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                     walk = true;
                 }
             }
-            finish_leaf<BF16>(S, R, e);
+            finish_leaf<BF16>(S, R, v, e);
             if (COUNT) {
                 if (kind == kMain) cnt[C_FLIGHTS]++;
                 else cnt[C_SUN_RAYS]++;
@@ -787,67 +832,64 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                     float wdt;
                     st = cross_face(S, R, p, nv, &wdt);
                     if (TERRAIN) { tg -= wdt; tpend -= wdt; }   // a periodic wrap restarts the segment
-                    if (st == kInside) e = __ldg(leaf_entry(S, R.v));
+                    if (st == kInside) e = __ldg(leaf_entry(S, nv));
                 }
                 // the block of a tentative collision, or of the roulette at a leaf
                 // crossing of decomposition tracking (word 3, which uses it up)
-                float k = R.M;
-                float ratio = 0.0f;
                 const bool roulette = DECOMP && decomp && face && st == kInside && Ts < 0.1f;
-                bool need = roulette;
-                if (COUNT && tent) ++tents;
+                const bool loads = tent && R.msk != 0;
+                float k = R.M;
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                if (loads || roulette) {
+                    if (!DECOMP || loads) {
+                        const size_t idx = brick_index(S, nv[0], nv[1], nv[2]);
+                        k = BF16 ? __uint_as_float((uint32_t)__ldg(S.vox16 + idx) << 16) : __ldg(S.vox + idx);
+                        k = __fadd_rn(k, S.k_gas);
+                    }
+                    const uint32_t ev = geti(K_EV) & ~kTermAfter;
+                    x = draw_block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk,
+                                   BATCH ? P.items[geti(K_CELL)].key : P.key);
+                    ++blk;
+                }
                 if (tent) {
                     if (COUNT) {
+                        ++tents;
                         if (kind == kMain) cnt[C_TENT]++;
                         else cnt[C_SUN_TENT]++;
                     }
                     R.t = tn;
-                    if (R.msk != 0) {
-                        // (a voxel leaf's majorant is the voxel itself: no load)
-                        const size_t idx = brick_index(S, nv[0], nv[1], nv[2]);
-                        k = BF16 ? __uint_as_float((uint32_t)__ldg(S.vox16 + idx) << 16) : __ldg(S.vox + idx);
-                        k = __fadd_rn(k, S.k_gas);
-                        need = true;
-                    }
-                    if (kind != kMain && P.sun_mode != MCRT_SUN_DELTA) {
-                        if (decomp) ratio = 1.0f - __fdividef(k - R.mn, R.M - R.mn);
-                        else ratio = 1.0f - __fdividef(k, R.M);
-                        // (0 in a voxel leaf but for rounding)
-                        need = need || ratio > 0.0f;
-                    }
-                }
-                uint4 x = make_uint4(0u, 0u, 0u, 0u);
-                if (need) {
-                    const uint32_t ev = geti(K_EV) & ~kTermAfter;
-                    x = draw_block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk,
-                                   BATCH ? P.items[geti(K_CELL)].key : P.key);
-                }
-                if (tent) {
-                    if (need) ++blk;
                     const float u0 = u01(x.x);
                     if (kind == kMain) {
-                        if (u0 * R.M <= k) {
+                        // (in a voxel leaf k is the majorant: real)
+                        if (!loads || u0 * R.M <= k) {
                             F(K_VX) = p[0]; F(K_VY) = p[1]; F(K_VZ) = p[2];
                             F(K_VK) = k;
                             phase = PH_VERTEX;
                             if constexpr (LEARNED) {
                                 if (geti(K_LV) < (uint32_t)P.n_learned) {
                                     phase = PH_SUSPEND;
-                                    R.v[0] = nv[0]; R.v[1] = nv[1]; R.v[2] = nv[2];
+                                    seti(K_NX, (uint32_t)nv[0]); seti(K_NY, (uint32_t)nv[1]); seti(K_NZ, (uint32_t)nv[2]);
                                 }
                             }
                         }
                     } else if (P.sun_mode == MCRT_SUN_DELTA) {
-                        if (u0 * R.M <= k) { Ts = 0.0f; phase = PH_SUN_END; }
+                        if (!loads || u0 * R.M <= k) { Ts = 0.0f; phase = PH_SUN_END; }
                     } else {
-                        Ts *= ratio;
-                        if (!(Ts > 0.0f)) { Ts = 0.0f; phase = PH_SUN_END; }
-                        else if (Ts < 0.1f) {
-                            if (u0 * 0.1f <= Ts) Ts = 0.1f;
+                        Ts *= decomp ? null_share<!EXTRA>(k - R.mn, R.M - R.mn) : null_share<!EXTRA>(k, R.M);
+                        if (!(Ts > 0.0f)) {
+                            Ts = 0.0f;
+                            phase = PH_SUN_END;
+                        } else if (Ts < 0.1f) {
+                            // (in a voxel leaf 1 - k/M is 0 or a rounding residual,
+                            // whose roulette waits for the rare pass)
+                            if (!loads) phase = PH_ROULETTE;
+                            else if (u0 * 0.1f <= Ts) Ts = 0.1f;
                             else { Ts = 0.0f; phase = PH_SUN_END; }
+                        } else if (!loads) {
+                            phase = PH_ROULETTE;
                         }
                     }
-                    if (phase == PH_STEP) tau = -__logf(u01(x.y));
+                    if (loads && phase == PH_STEP) tau = -__logf(u01(x.y));
                 } else if (at_ground) {
                     // ground vertex at the surface hit (x, y wrapped into the domain)
 #pragma unroll
@@ -860,7 +902,6 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                     phase = PH_GROUND;
                 } else if (st == kInside) {
                     if (roulette) {
-                        ++blk;
                         if (u01(x.w) * 0.1f <= Ts) Ts = 0.1f;
                         else { Ts = 0.0f; phase = PH_SUN_END; }
                     }
@@ -869,7 +910,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                             if (kind == kMain) cnt[C_LEAF]++;
                             else cnt[C_SUN_LEAF]++;
                         }
-                        finish_leaf<BF16>(S, R, e);
+                        finish_leaf<BF16>(S, R, nv, e);
                         if (R.steps > P.max_steps) {
                             if (COUNT) cnt[C_ABORT]++;
                             Ts = 0.0f;
@@ -897,7 +938,8 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         mark(4);
     }
 
-    // ---- partial sums left by a deadline / cancel exit ------------------------
+    // ---- the warp's sums, and partial ones left by a deadline / cancel exit ----
+    spill_sums();
     if (phase != PH_IDLE && phase != PH_CLAIM) {
 #pragma unroll
         for (int q = 0; q < 2 * NQ; ++q)
@@ -961,18 +1003,19 @@ __global__ void debug_dda_kernel(DevScene S, float ox, float oy, float oz, float
         if (n >= cap) { status = 3; break; }
         const int lev = __popc((unsigned)R.msk);
         cells[4 * n + 0] = lev / S.lb;        // level of the tracked grid
-        cells[4 * n + 1] = R.v[0] >> lev;
-        cells[4 * n + 2] = R.v[1] >> lev;
-        cells[4 * n + 3] = R.v[2] >> lev;
+        cells[4 * n + 1] = R.lo[0] >> lev;
+        cells[4 * n + 2] = R.lo[1] >> lev;
+        cells[4 * n + 3] = R.lo[2] >> lev;
         tio[2 * n + 0] = __fadd_rn(tbase, R.t);
         tio[2 * n + 1] = __fadd_rn(tbase, R.texit);
         ++n;
         float wdt, p[3];
-        const int st = step_face(S, R, p, &wdt);
+        int v[3];
+        const int st = step_face(S, R, p, v, &wdt);
         if (wdt != 0.0f) tbase = __fadd_rn(tbase, wdt);
         if (st == kTop) { status = 1; break; }
         if (st == kGround) { status = 2; break; }
-        finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+        finish_leaf<BF16>(S, R, v, __ldg(leaf_entry(S, v)));
         if (R.steps > (1u << 22)) { status = 4; break; }
     }
     count_status[0] = n;
@@ -1028,9 +1071,10 @@ __global__ void view_cost_kernel(TraceParams P, int tiles_x, int tiles_y, float*
         for (int n = 0; n < 4096 && c < 1e4f; ++n) {
             c += R.M * (R.texit - R.t);
             float wdt, p[3];
-            const int st = step_face(S, R, p, &wdt);
+            int v[3];
+            const int st = step_face(S, R, p, v, &wdt);
             if (st != kInside) break;
-            finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+            finish_leaf<BF16>(S, R, v, __ldg(leaf_entry(S, v)));
         }
     }
     cost[i] = c;

@@ -125,16 +125,7 @@ __device__ __forceinline__ void wf_tally(const TraceParams& P, uint32_t cell, fl
 template <bool BF16>
 __device__ __forceinline__ void wf_ray_start(const DevScene& S, Ray& R, const float o[3], const float d[3])
 {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        R.o[a] = o[a];
-        R.d[a] = d[a];
-        R.inv_d[a] = dir_rcp(d[a]);
-        R.v[a] = locate(o[a], d[a], S.h[a], S.inv_h[a], 0, S.n[a] - 1);
-    }
-    R.t = 0.0f;
-    R.steps = 0;
-    finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+    ray_begin<BF16>(S, R, o, d);
 }
 
 // A stage kernel's threads are persistent: a lane that finishes its entry
@@ -187,7 +178,7 @@ __device__ __forceinline__ bool wf_step(const DevScene& S, Ray& R, float& tau, f
     tau -= Mseg;
     float wdt;
     *st = cross_face(S, R, p, nv, &wdt);
-    if (*st == kInside) finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+    if (*st == kInside) finish_leaf<BF16>(S, R, nv, __ldg(leaf_entry(S, nv)));
     return false;
 }
 
@@ -226,18 +217,19 @@ __global__ void __launch_bounds__(kWfBlock) wf_flight_kernel(const __grid_consta
                 blk = 1;
             } else {
                 // a flight suspended at its step budget: re-entering its
-                // leaf from the same voxel at the same distance gives the
+                // leaf (by its first voxel) at the same distance gives the
                 // same leaf, majorant and exit as before
+                int v[3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     R.o[a] = o[a];
                     R.d[a] = d[a];
                     R.inv_d[a] = dir_rcp(d[a]);
-                    R.v[a] = (int)F.vox[a][i];
+                    v[a] = (int)F.vox[a][i];
                 }
                 R.t = F.t[i];
                 R.steps = F.steps[i];
-                finish_leaf<BF16>(S, R, __ldg(leaf_entry(S, R.v)));
+                finish_leaf<BF16>(S, R, v, __ldg(leaf_entry(S, v)));
             }
             budget = kStepsPerRound;
             have = true;
@@ -293,7 +285,7 @@ __global__ void __launch_bounds__(kWfBlock) wf_flight_kernel(const __grid_consta
                 wf_put(G, gslot, pid, cell, ev, 0u, w, score, R.o, R.d, tau);
                 G.blk[gslot] = blk;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) G.vox[a][gslot] = (uint32_t)R.v[a];
+                for (int a = 0; a < 3; ++a) G.vox[a][gslot] = (uint32_t)R.lo[a];
                 G.t[gslot] = R.t;
                 G.steps[gslot] = R.steps;
             } else {
@@ -387,7 +379,7 @@ __global__ void __launch_bounds__(kWfBlock) wf_vertex_kernel(const __grid_consta
                     if (P.sun_mode == MCRT_SUN_DELTA) {
                         if (u0 * R.M <= k) { Ts = 0.0f; ended = true; }
                     } else {
-                        Ts *= 1.0f - __fdividef(k, R.M);
+                        Ts *= null_share<true>(k, R.M);
                         if (!(Ts > 0.0f)) {
                             Ts = 0.0f;
                             ended = true;
