@@ -759,6 +759,7 @@ int run_trace(mcrt_scene* sc, TraceParams& P, int sensor, const mcrt_trace_opts*
     P.sun_mode = o->sun_mode;
     P.max_steps = 1u << 22;
     set_rare_batch(P, o->rare_batch);
+    set_claim_lanes(P, grid, block);
     cudaEvent_t e0, e1;
     CK(ctx, cudaEventCreate(&e0));
     CK(ctx, cudaEventCreate(&e1));
@@ -888,6 +889,7 @@ int run_learned(mcrt_scene* sc, const TraceParams& P0, int sensor, const mcrt_tr
             P.qin = qin; P.qin_feat = fin_feat; P.qin_mix = mix;
             P.qout = qout; P.qout_feat = fout; P.qout_count = cnt; P.qout_cap = (unsigned)nb;
             if (P.total == 0) break;
+            set_claim_lanes(P, grid, block);
             if (r > 0) {
                 ctx->launches++;
                 e = launch_mlp_infer(prop->d_wbf, prop->d_bias, fin_feat, (int)n_in, mix, nullptr, ctx->sm_count,
@@ -1275,9 +1277,10 @@ int mcrt_trace_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, con
     CK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_items), sizeof(BatchItem) * (size_t)n, ctx->stream));
     cudaError_t e = cudaMemcpyAsync(d_items, h.data(), sizeof(BatchItem) * (size_t)n, cudaMemcpyHostToDevice,
                                     ctx->stream);
-    const TraceParams P = batch_params(h, d_items, total, o, t);
+    TraceParams P = batch_params(h, d_items, total, o, t);
     int block = 0;
     const int grid = batch_grid(ctx, o, bf16, &block);
+    set_claim_lanes(P, grid, block);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -1424,9 +1427,10 @@ int mcrt_batch_plan_create(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t 
                     cudaGetErrorString(e));
     }
     mcrt_tally* t = p->t;
-    const TraceParams P = batch_params(p->h, p->d_items, total, o, t);
+    TraceParams P = batch_params(p->h, p->d_items, total, o, t);
     int block = 0;
     const int grid = batch_grid(ctx, o, bf16, &block);
+    set_claim_lanes(P, grid, block);
     e = cudaStreamBeginCapture(p->st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t c = cudaMemsetAsync(t->d_s1, 0, m * sizeof(double), p->st);

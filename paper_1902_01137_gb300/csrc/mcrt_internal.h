@@ -150,6 +150,7 @@ struct TraceParams {
     uint32_t max_steps;
     int rare_batch;            // lanes waiting for a rare phase that trigger it
     int min_steppers;          // below this many stepping lanes, run rare phases anyway
+    int claim_lanes;           // lanes of a warp that claim paths; the others only help
     // camera
     int width, height;
     uint32_t spp;
@@ -211,6 +212,17 @@ inline void set_rare_batch(TraceParams& P, int requested)
 {
     P.rare_batch = requested > 0 ? requested : kDefaultRareBatch;
     P.min_steppers = 33 - P.rare_batch;
+}
+
+// Lanes of a warp that claim paths: all 32 when there are claims for every
+// resident lane, else the claims spread evenly over the warps, and the lanes
+// left over help from the start.  Launch shape only.
+inline void set_claim_lanes(TraceParams& P, int grid, int block)
+{
+    const unsigned long long warps = (unsigned long long)grid * (unsigned)(block / 32);
+    const unsigned long long claims = (P.total + P.chunk - 1) / P.chunk;
+    const unsigned long long per = warps ? (claims + warps - 1) / warps : 32ull;
+    P.claim_lanes = per >= 32 ? 32 : (per < 1 ? 1 : (int)per);
 }
 
 enum Sensor { kCamera = 0, kFlux = 1 };
