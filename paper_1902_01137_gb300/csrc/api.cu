@@ -1038,7 +1038,7 @@ int mcrt_trace_camera(mcrt_scene* sc, const mcrt_camera_desc* cam, uint32_t spp,
     if (chunk > spp) chunk = spp;
     while (spp % chunk) --chunk;   // a chunk never straddles two pixels
     P.chunk = chunk;
-    P.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    set_key(P, seed);
     P.width = cam->width;
     P.height = cam->height;
     P.spp = spp;
@@ -1125,7 +1125,7 @@ int mcrt_trace_flux(mcrt_scene* sc, uint64_t npaths, uint64_t seed, const mcrt_t
     P.S = make_dev_scene(sc, 0.0f);
     P.total = npaths;
     P.chunk = o->chunk ? (uint32_t)o->chunk : 4u;
-    P.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    set_key(P, seed);
     P.spp = 1;
     P.Lz = (float)sc->n[2] * sc->h[2];
     if (o->proposal) {

@@ -61,6 +61,21 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
     return c;
 }
 
+// The same with the ten rounds' keys laid out beforehand (a launch's one key,
+// read as constants: 18 additions of 64 instructions less).
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const uint2 (&ks)[10])
+{
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
+        const uint32_t lo0 = 0xD2511F53u * c.x;
+        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
+        const uint32_t lo1 = 0xCD9E8D57u * c.z;
+        c = make_uint4(hi1 ^ c.y ^ ks[r].x, lo1, hi0 ^ c.w ^ ks[r].y, lo0);
+    }
+    return c;
+}
+
 // Random numbers are addressed: stream s of event e of path p evaluates
 // Philox at counter (p lo, p hi, (e << 2) | s, block) and uses fixed words of
 // the block -- block 0 word 0: first optical depth of a flight or a flux

@@ -144,7 +144,8 @@ struct TraceParams {
     DevScene S;
     unsigned long long total;  // paths
     uint32_t chunk;            // paths per claim
-    uint2 key;                 // Philox key (seed)
+    uint2 key;                 // Philox key (seed) ...
+    uint2 ks[10];              // ... and its rounds' keys
     int max_order;
     int sun_mode;
     uint32_t max_steps;
@@ -212,6 +213,12 @@ inline void set_rare_batch(TraceParams& P, int requested)
 {
     P.rare_batch = requested > 0 ? requested : kDefaultRareBatch;
     P.min_steppers = 33 - P.rare_batch;
+}
+
+inline void set_key(TraceParams& P, uint64_t seed)
+{
+    P.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    for (uint32_t r = 0; r < 10; ++r) P.ks[r] = make_uint2(P.key.x + r * 0x9E3779B9u, P.key.y + r * 0xBB67AE85u);
 }
 
 // Lanes of a warp that claim paths: all 32 when there are claims for every

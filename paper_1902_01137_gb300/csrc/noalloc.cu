@@ -158,7 +158,7 @@ extern "C" int mcrt_trace_camera_noalloc(mcrt_scene* sc, const mcrt_camera_desc*
     if (chunk > spp) chunk = spp;
     while (spp % chunk) --chunk;
     P.chunk = chunk;
-    P.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    set_key(P, seed);
     P.width = cam->width;
     P.height = cam->height;
     P.spp = spp;
