@@ -482,7 +482,8 @@ int mcrt_scene_set_ground_flat(mcrt_scene* sc, float albedo)
     sc->albedo = albedo;
     dfree(sc->ctx, sc->d_hf);
     dfree(sc->ctx, sc->d_hpyr);
-    sc->d_hf = sc->d_hpyr = nullptr;
+    sc->d_hf = nullptr;
+    sc->d_hpyr = nullptr;
     sc->hlev = 0;
     sc->gen++;
     return MCRT_OK;
@@ -512,9 +513,11 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     }
     const size_t n = (size_t)hnx * hny;
     float *dh = nullptr, *dp = nullptr;
+    float4* dc = nullptr;
     int* bad = nullptr;
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&dh), n * sizeof(float), ctx->stream);
     if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&dp), total * sizeof(float), ctx->stream);
+    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&dc), n * sizeof(float4), ctx->stream);
     if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&bad), sizeof(int), ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(dh, heights, n * sizeof(float),
@@ -522,7 +525,7 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream);
     const float top = (float)sc->n[2] * sc->h[2];
     if (e == cudaSuccess) { ctx->launches++; e = launch_hf_check(dh, (long long)n, top, bad, ctx->stream); }
-    if (e == cudaSuccess) { ctx->launches += lev; e = launch_hf_pyramid(dh, hnx, hny, dp, off, lev, ctx->stream); }
+    if (e == cudaSuccess) { ctx->launches += lev; e = launch_hf_pyramid(dh, hnx, hny, dc, dp, off, lev, ctx->stream); }
     const size_t ntop = (size_t)(hnx >> (2 * (lev - 1))) * (size_t)(hny >> (2 * (lev - 1)));
     std::vector<float> tops(ntop);
     int hbad = 0;
@@ -530,16 +533,17 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(tops.data(), dp + off[lev - 1], ntop * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);
     if (bad) cudaFreeAsync(bad, ctx->stream);
+    dfree(ctx, dh);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess || hbad) {
-        dfree(ctx, dh);
+        dfree(ctx, dc);
         dfree(ctx, dp);
         if (e != cudaSuccess) return fail(ctx, MCRT_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
         return fail(ctx, MCRT_ERR_ARG, "%s: heights must be finite and in [0, %g] km", who, (double)top);
     }
     dfree(ctx, sc->d_hf);
     dfree(ctx, sc->d_hpyr);
-    sc->d_hf = dh;
+    sc->d_hf = dc;
     sc->d_hpyr = dp;
     sc->hn[0] = hnx;
     sc->hn[1] = hny;

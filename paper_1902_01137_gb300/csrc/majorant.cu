@@ -308,20 +308,24 @@ cudaError_t launch_octree(const mcrt_scene* sc, const DevScene& S, cudaStream_t 
 
 // ---------------------------------------------------------------------------
 // Heightfield ground: max pyramid.  Level 0 holds each cell's maximum over
-// its 4 corner heights (periodic); level L the maximum over 4 x 4 cells of
+// its 4 corner heights (periodic), which are kept as one record per cell;
+// level L the maximum over 4 x 4 cells of
 // level L - 1.  Also a scan for invalid heights (not finite, < 0 or above
 // the top of the field).
 // ---------------------------------------------------------------------------
 namespace {
 
-__global__ void hf_cellmax_kernel(const float* __restrict__ h, int nx, int ny, float* __restrict__ out)
+__global__ void hf_cellmax_kernel(const float* __restrict__ h, int nx, int ny, float4* __restrict__ cells,
+                                  float* __restrict__ out)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)nx * ny) return;
     const int i = (int)(idx % nx), j = (int)(idx / nx);
     const int i1 = i + 1 == nx ? 0 : i + 1, j1 = j + 1 == ny ? 0 : j + 1;
-    out[idx] = fmaxf(fmaxf(h[(size_t)j * nx + i], h[(size_t)j * nx + i1]),
-                     fmaxf(h[(size_t)j1 * nx + i], h[(size_t)j1 * nx + i1]));
+    const float4 c = make_float4(h[(size_t)j * nx + i], h[(size_t)j * nx + i1], h[(size_t)j1 * nx + i],
+                                 h[(size_t)j1 * nx + i1]);
+    cells[idx] = c;
+    out[idx] = fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w));
 }
 
 __global__ void hf_reduce4_kernel(const float* __restrict__ in, int nx, int ny, float* __restrict__ out)
@@ -347,10 +351,11 @@ __global__ void hf_check_kernel(const float* __restrict__ h, long long n, float 
 
 }  // namespace
 
-cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float* pyr, const int* off, int levels, cudaStream_t st)
+cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float4* cells, float* pyr, const int* off, int levels,
+                              cudaStream_t st)
 {
     const long long n0 = (long long)nx * ny;
-    hf_cellmax_kernel<<<(unsigned)((n0 + 255) / 256), 256, 0, st>>>(h, nx, ny, pyr + off[0]);
+    hf_cellmax_kernel<<<(unsigned)((n0 + 255) / 256), 256, 0, st>>>(h, nx, ny, cells, pyr + off[0]);
     for (int L = 1; L < levels; ++L) {
         const int px = nx >> (2 * (L - 1)), py = ny >> (2 * (L - 1));
         const long long n = (long long)(px >> 2) * (py >> 2);

@@ -124,10 +124,11 @@ struct DevScene {
     float inv_sun[3];    // its reciprocals as dir_rcp gives them
     int rayleigh;        // clear air scatters with the Rayleigh phase function (else HG with g)
     // heightfield ground (hf null: flat ground at z = 0).  Heights sit at
-    // the corners of a periodic grid of hn[0] x hn[1] cells; hpyr holds the
-    // cell maxima (level 0: max of a cell's 4 corners) and hlev - 1 coarser
+    // the corners of a periodic grid of hn[0] x hn[1] cells; hf holds each
+    // cell's four, (i, j), (i+1, j), (i, j+1), (i+1, j+1), hpyr the cell
+    // maxima (level 0: max of a cell's 4 corners) and hlev - 1 coarser
     // levels of 4 x 4 blocks, concatenated at hoff[level].
-    const float* __restrict__ hf;
+    const float4* __restrict__ hf;
     const float* __restrict__ hpyr;
     int hn[2];
     float hc[2];         // cell size [km]
@@ -445,17 +446,19 @@ __device__ __forceinline__ int hf_wrap(const DevScene& S, int a, int i, int L)
 }
 
 // The 4 corner heights of cell (i, j): h[0] = (i, j), h[1] = (i+1, j),
-// h[2] = (i, j+1), h[3] = (i+1, j+1).
+// h[2] = (i, j+1), h[3] = (i+1, j+1).  One record per cell: a walk is a chain
+// of dependent loads, and this one gives the cell's corners and its maximum
+// together (from the plain height grid they were two loads behind each
+// other, the second of four words in two rows).
 __device__ __forceinline__ void hf_corners(const DevScene& S, int i, int j, float h[4])
 {
-    const int i0 = hf_wrap(S, 0, i, 0), i1 = hf_wrap(S, 0, i + 1, 0);
-    const size_t r0 = (size_t)hf_wrap(S, 1, j, 0) * S.hn[0], r1 = (size_t)hf_wrap(S, 1, j + 1, 0) * S.hn[0];
-    MCRT_CHECK(i0 >= 0 && i0 < S.hn[0] && i1 >= 0 && i1 < S.hn[0] && r0 < (size_t)S.hn[0] * S.hn[1] &&
-                   r1 < (size_t)S.hn[0] * S.hn[1], 4);
-    h[0] = __ldg(S.hf + r0 + i0);
-    h[1] = __ldg(S.hf + r0 + i1);
-    h[2] = __ldg(S.hf + r1 + i0);
-    h[3] = __ldg(S.hf + r1 + i1);
+    const int i0 = hf_wrap(S, 0, i, 0), j0 = hf_wrap(S, 1, j, 0);
+    MCRT_CHECK(i0 >= 0 && i0 < S.hn[0] && j0 >= 0 && j0 < S.hn[1], 4);
+    const float4 c = __ldg(S.hf + ((unsigned long long)(uint32_t)j0 * (uint32_t)S.hn[0] + (uint32_t)i0));
+    h[0] = c.x;
+    h[1] = c.y;
+    h[2] = c.z;
+    h[3] = c.w;
 }
 
 __device__ __forceinline__ void hf_plane(const float h[4], bool triA, float* a, float* b, float* c)
@@ -539,7 +542,13 @@ __device__ __forceinline__ bool terrain_walk_step(const DevScene& S, const float
     const int nx = S.hn[0] >> sh;
     MCRT_CHECK(W.L >= 0 && W.L < S.hlev && hf_wrap(S, 0, W.i, W.L) < nx && hf_wrap(S, 1, W.j, W.L) < (S.hn[1] >> sh) &&
                    hf_wrap(S, 0, W.i, W.L) >= 0 && hf_wrap(S, 1, W.j, W.L) >= 0, 5);
-    const float cmax = __ldg(S.hpyr + S.hoff[W.L] + (size_t)hf_wrap(S, 1, W.j, W.L) * nx + hf_wrap(S, 0, W.i, W.L));
+    float hc4[4], cmax;
+    if (W.L == 0) {
+        hf_corners(S, W.i, W.j, hc4);
+        cmax = fmaxf(fmaxf(hc4[0], hc4[1]), fmaxf(hc4[2], hc4[3]));
+    } else {
+        cmax = __ldg(S.hpyr + S.hoff[W.L] + (size_t)hf_wrap(S, 1, W.j, W.L) * nx + hf_wrap(S, 0, W.i, W.L));
+    }
     const float zlo = __fmaf_rn(d[2] < 0.0f ? te : W.t, d[2], o[2]);
     if (zlo <= cmax) {
         if (W.L > 0) {
@@ -565,8 +574,6 @@ __device__ __forceinline__ bool terrain_walk_step(const DevScene& S, const float
             const float tm = __fdividef(-g0, g1);
             if (tm > W.t && tm < te) { cut1 = tm; np = 2; }
         }
-        float hc4[4];
-        hf_corners(S, W.i, W.j, hc4);
         for (int q = 0; q < np; ++q) {
             const float a0 = q == 0 ? W.t : cut1, b0 = q == 0 ? cut1 : te;
             const bool triA = __fmaf_rn(g1, 0.5f * (a0 + b0), g0) >= 0.0f;

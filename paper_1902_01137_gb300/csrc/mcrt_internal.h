@@ -82,7 +82,7 @@ struct mcrt_scene {
     float sun_zenith = 0, sun_azimuth = 0;
     float sun[3] = {0, 0, 1};
     // heightfield ground (null: flat)
-    float* d_hf = nullptr;
+    float4* d_hf = nullptr;
     float* d_hpyr = nullptr;
     int hn[2] = {0, 0};
     float hmax = 0;
@@ -208,10 +208,12 @@ struct TraceParams {
 // runs half empty: cumulus image of 16.8 M paths 62.1, 57.3, 56.3, 57.9,
 // 64.2 ms at 8, 12, 16, 20, 24 lanes; flux of the same field 53.3, 51.7,
 // 49.9, 48.3, 52.1 ms; octree image 35.2, 32.8, 32.3, 32.9, 35.3 ms.
-constexpr int kDefaultRareBatch = 16;
+// Over a heightfield, where a pass costs more (and walkers wait besides): 20.0,
+// 19.6, 19.3, 19.2 ms at 16, 18, 20, 22.
+constexpr int kDefaultRareBatch = 16, kDefaultRareBatchHf = 20;
 inline void set_rare_batch(TraceParams& P, int requested)
 {
-    P.rare_batch = requested > 0 ? requested : kDefaultRareBatch;
+    P.rare_batch = requested > 0 ? requested : (P.S.hf ? kDefaultRareBatchHf : kDefaultRareBatch);
     P.min_steppers = 33 - P.rare_batch;
 }
 
@@ -240,7 +242,8 @@ cudaError_t launch_reduce_level(const float* prev, const int* prev_dims, float* 
                                 cudaStream_t st);
 cudaError_t launch_leafmap(const mcrt_scene* sc, float tau, int finest, int grid, cudaStream_t st);
 cudaError_t launch_octree(const mcrt_scene* sc, const DevScene& S, cudaStream_t st);
-cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float* pyr, const int* off, int levels, cudaStream_t st);
+cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float4* cells, float* pyr, const int* off, int levels,
+                              cudaStream_t st);
 cudaError_t launch_hf_check(const float* h, long long n, float top, int* bad, cudaStream_t st);
 cudaError_t launch_debug_terrain(const DevScene& S, const float* o, const float* d, int n, float* t, cudaStream_t st);
 cudaError_t launch_debug_terrain_height(const DevScene& S, const float* xy, int n, float* zn, cudaStream_t st);

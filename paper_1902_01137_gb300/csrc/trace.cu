@@ -98,7 +98,7 @@ enum Phase {
     PH_GROUND,      // a ground vertex
     PH_RESUME,      // a path stopped at a learned vertex goes on
     PH_SUSPEND,     // a path stops at a learned vertex
-    PH_TERRAIN,     // a flight reached the relief layer: find its ground hit
+    PH_WALK,        // the ray's hit on the heightfield is to be found
     PH_HIT,         // a tentative collision in a voxel leaf, at distance R.t
     PH_ROULETTE,    // ... that left a sun ray a residual Ts: its draw
     PH_REAL,        // a real collision at distance R.t of extinction K_VK
@@ -124,6 +124,12 @@ enum Cold {
     K_DONE = K_LEFT, K_WORD = K_NX, K_TS = K_SCORE
 };
 constexpr uint32_t kTermAfter = 0x80000000u;   // the path ends with this event's estimate
+// Heightfield walkers of a warp that go together.  A path walks about three
+// times, so a pass rarely has two walkers, and each walk alone held the warp
+// for some twenty dependent loads: 4 M flux paths over a 4096^2 relief 23.7
+// ms with each walk at once, 20.9 ms in eights (21.6 in fours, 21.4 in
+// twelves), 20.0 ms with a cell's corners in one record.
+constexpr int kWalkBatch = 8;
 // K_Q: the number of helpers at work (low 3 bits), then their lanes, first
 // handed off first, 5 bits each.
 constexpr uint32_t kMaxHelpers = 5;
@@ -568,7 +574,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 }
             }
         }
-        bool ran = phase >= PH_CLAIM;
+        bool ran = phase >= PH_CLAIM && !(TERRAIN && phase == PH_WALK);
         if (COUNT) {
             if (ran) ++path_iters;
             const unsigned rr = __ballot_sync(kFull, ran);
@@ -613,7 +619,6 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         const unsigned long long pid = get_pid();
         bool begin = phase == PH_BEGIN;   // start a ray now ...
         uint32_t tw = 0u;                 // ... whose first optical depth comes from this word
-        bool walk = false;                // heightfield: find this ray's ground hit now
         float vx[3] = {0.0f, 0.0f, 0.0f}, nd[3] = {0.0f, 0.0f, 0.0f};
         uint4 x = make_uint4(0u, 0u, 0u, 0u);
         if (ran) {
@@ -940,17 +945,14 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
             blk = 1;
             phase = PH_STEP;
             if constexpr (TERRAIN) {
-                // a sun ray that meets the surface is shadowed (found now: sun rays
-                // only start inside the relief layer at the ground or below hmax);
-                // a flight ends at the surface, found now when it starts inside the
-                // relief layer, else once its traversal reaches z = hmax
+                // a sun ray that meets the surface is shadowed (only one that starts
+                // inside the relief layer can); a flight ends at the surface, found
+                // first when it starts inside the relief layer, else once its
+                // traversal reaches z = hmax
                 tg = kInf;
                 tpend = kInf;
-                if (kind == kMain && R.o[2] > Z.hmax) {
-                    if (R.d[2] < 0.0f) tpend = __fdiv_rn(Z.hmax - R.o[2], R.d[2]);
-                } else {
-                    walk = true;
-                }
+                if (!(R.o[2] > Z.hmax)) phase = PH_WALK;
+                else if (kind == kMain && R.d[2] < 0.0f) tpend = __fdiv_rn(Z.hmax - R.o[2], R.d[2]);
             }
             finish_leaf<BF16>(Z, R, v, e);
             if (COUNT) {
@@ -959,18 +961,20 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
             }
         }
         if constexpr (TERRAIN) {
-            if (phase == PH_TERRAIN) {
-                walk = true;
-                tpend = kInf;
-                phase = PH_STEP;
-            }
-            if (walk) {
-                const float th = terrain_hit(Z, R.o, R.d);
-                if (kind == kMain) {
-                    tg = th;
-                } else if (th < kInf) {
-                    Ts = 0.0f;
-                    phase = PH_SUN_END;
+            // ---- walks over the heightfield wait until kWalkBatch lanes walk
+            //      together or too few lanes step to wait any longer -----------------
+            const unsigned walkers = __ballot_sync(kFull, phase == PH_WALK);
+            const int steppers = __popc(__ballot_sync(kFull, phase == PH_STEP));
+            if (__popc(walkers) >= kWalkBatch || (walkers && steppers < P.min_steppers)) {
+                if (phase == PH_WALK) {
+                    const float th = terrain_hit(Z, R.o, R.d);
+                    phase = PH_STEP;
+                    if (kind == kMain) {
+                        tg = th;
+                    } else if (th < kInf) {
+                        Ts = 0.0f;
+                        phase = PH_SUN_END;
+                    }
                 }
             }
         }
@@ -982,7 +986,10 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         do {
             // (heightfield: a flight whose current leaf reaches down into the relief
             //  layer first finds its ground hit, in a rare pass)
-            if (TERRAIN && phase == PH_STEP && R.texit >= tpend) phase = PH_TERRAIN;
+            if (TERRAIN && phase == PH_STEP && R.texit >= tpend) {
+                phase = PH_WALK;
+                tpend = kInf;
+            }
             if (COUNT) {
                 const unsigned st = __ballot_sync(kFull, phase == PH_STEP), lv = __ballot_sync(kFull, phase != PH_IDLE);
                 occ[0] += 1; occ[1] += __popc(lv); occ[2] += __popc(st); occ[5] += __popc(lv) - __popc(st);
