@@ -183,6 +183,11 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
         seti(K_PID_HI, (uint32_t)(pid >> 32));
     };
 
+    // score + cf T: one operation, or two (a batch's other sums use the
+    // product); each variant keeps the rounding it has always had
+    auto add_estimate = [](float score, float cf, float T) -> float {
+        return BATCH ? __fadd_rn(score, __fmul_rn(cf, T)) : __fmaf_rn(cf, T, score);
+    };
     auto block = [&](unsigned long long pid, uint32_t c2, uint32_t b) -> uint4 {
         if constexpr (BATCH) return draw_block(pid, c2, b, P.items[geti(K_CELL)].key);
         else return philox4x32_10(make_uint4((uint32_t)pid, (uint32_t)(pid >> 32), c2, b), P.ks);
@@ -322,7 +327,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 const int h = (tid & ~31) + (int)((q >> 3) & 31u);
                 if (__float_as_uint(cold[K_DONE][h]) != 1u) break;
                 const float cf = cold[K_CF][h], hT = cold[K_TS][h];
-                F(K_SCORE) = __fmaf_rn(cf, hT, F(K_SCORE));
+                F(K_SCORE) = add_estimate(F(K_SCORE), cf, hT);
                 if constexpr (BATCH) {
                     const float e = __fmul_rn(cf, hT);
                     F(K_DSC) = __fmaf_rn(e, cold[K_CFS][h], F(K_DSC));
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
                 phase = PH_BEGIN;
             } else {
                 const float cf = F(K_CF);
-                F(K_SCORE) = __fmaf_rn(cf, Ts, F(K_SCORE));
+                F(K_SCORE) = add_estimate(F(K_SCORE), cf, Ts);
                 if constexpr (BATCH) {
                     const float e = __fmul_rn(cf, Ts);
                     F(K_DSC) = __fmaf_rn(e, F(K_SG) + F(K_CFS), F(K_DSC));
