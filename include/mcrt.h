@@ -597,9 +597,11 @@ MCRT_API int mcrt_debug_terrain_height(const mcrt_scene* scene, int32_t n, const
 MCRT_API int mcrt_debug_bounds_violations(mcrt_ctx* ctx, int32_t* checked_build, uint64_t* count,
                                           int32_t* first_code);
 
-/* Device memory held by the allocations of the context's device's current
- * stream-ordered memory pool (the pool every allocation of this library
- * draws from, except a batch plan's item table): *used_current now and
+/* Device memory held by the allocations of the library's stream-ordered
+ * memory pool on the context's device (the pool every allocation of this
+ * library draws from, except a batch plan's item table; shared by the
+ * device's contexts, destroyed with the last, and keeping at most 4 GiB that
+ * nothing uses): *used_current now and
  * *used_high the most since the last reset; reset_high != 0 then resets the
  * high mark to the current use.  Lets a caller check that a call allocated
  * nothing (the paper has no counterpart).  Synchronises the context

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <mutex>
 #include <new>
 #include <vector>
 #include <utility>
@@ -49,7 +50,7 @@ int fail(mcrt_ctx* ctx, int code, const char* fmt, ...)
 template <class T>
 cudaError_t dalloc(mcrt_ctx* ctx, T** p, size_t bytes)
 {
-    return cudaMallocAsync(reinterpret_cast<void**>(p), bytes == 0 ? 16 : bytes, ctx->stream);
+    return pool_alloc(ctx, p, bytes);
 }
 
 void dfree(mcrt_ctx* ctx, void* p)
@@ -72,6 +73,58 @@ bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
 }  // namespace
 
 namespace mcrt {
+
+namespace {
+
+constexpr int kMaxPools = 64;
+std::mutex g_pool_mu;
+struct { cudaMemPool_t pool; int refs; } g_pools[kMaxPools];
+
+}  // namespace
+
+cudaError_t pool_acquire(int device, cudaMemPool_t* pool)
+{
+    if (device >= kMaxPools) return cudaDeviceGetDefaultMemPool(pool, device);
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    auto& g = g_pools[device];
+    if (g.refs == 0) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaError_t e = cudaMemPoolCreate(&g.pool, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t never = UINT64_MAX;             // pool_trim gives memory back
+        e = cudaMemPoolSetAttribute(g.pool, cudaMemPoolAttrReleaseThreshold, &never);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(g.pool);
+            return e;
+        }
+    }
+    ++g.refs;
+    *pool = g.pool;
+    return cudaSuccess;
+}
+
+void pool_release(int device)
+{
+    if (device >= kMaxPools) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    auto& g = g_pools[device];
+    // (memory a caller never freed keeps the pool alive inside the driver)
+    if (g.refs > 0 && --g.refs == 0) cudaMemPoolDestroy(g.pool);
+}
+
+void pool_trim(cudaMemPool_t pool)
+{
+    uint64_t held = 0, used = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+    }
+    if (held > used + kPoolKeep && cudaMemPoolTrimTo(pool, (size_t)used + kPoolKeep) != cudaSuccess) (void)cudaGetLastError();
+}
 
 DevScene make_dev_scene(const mcrt_scene* sc, float k_gas)
 {
@@ -169,6 +222,12 @@ int mcrt_create(mcrt_ctx** out, int device, void* cuda_stream)
         return fail(nullptr, MCRT_ERR_CUDA, "mcrt_create: %s", cudaGetErrorString(e));
     }
     c->l2_bytes = (size_t)l2;
+    e = pool_acquire(device, &c->pool);
+    if (e != cudaSuccess) {
+        delete c;
+        return fail(nullptr, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "mcrt_create: memory pool: %s",
+                    cudaGetErrorString(e));
+    }
     *out = c;
     return MCRT_OK;
 }
@@ -177,6 +236,7 @@ int mcrt_destroy(mcrt_ctx* ctx)
 {
     if (!ctx) return fail(nullptr, MCRT_ERR_ARG, "mcrt_destroy: NULL context");
     cudaStreamSynchronize(ctx->stream);
+    pool_release(ctx->device);
     delete ctx;
     return MCRT_OK;
 }
@@ -296,6 +356,7 @@ int mcrt_scene_destroy(mcrt_scene* sc)
     dfree(ctx, sc->d_hf);
     dfree(ctx, sc->d_hpyr);
     cudaStreamSynchronize(ctx->stream);
+    pool_trim(ctx->pool);
     delete sc;
     return MCRT_OK;
 }
@@ -515,10 +576,10 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     float *dh = nullptr, *dp = nullptr;
     float4* dc = nullptr;
     int* bad = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&dh), n * sizeof(float), ctx->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&dp), total * sizeof(float), ctx->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&dc), n * sizeof(float4), ctx->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&bad), sizeof(int), ctx->stream);
+    cudaError_t e = dalloc(ctx, &dh, n * sizeof(float));
+    if (e == cudaSuccess) e = dalloc(ctx, &dp, total * sizeof(float));
+    if (e == cudaSuccess) e = dalloc(ctx, &dc, n * sizeof(float4));
+    if (e == cudaSuccess) e = dalloc(ctx, &bad, sizeof(int));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(dh, heights, n * sizeof(float),
                             mem == MCRT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, ctx->stream);
@@ -802,7 +863,7 @@ int run_wavefront(mcrt_scene* sc, TraceParams& P, const mcrt_trace_opts* o, mcrt
     if (slots > P.total) slots = P.total ? P.total : 1ull;
     WavefrontStats ws{};
     const cudaError_t e = wavefront_camera(P, sc->storage == MCRT_STORAGE_BF16, (unsigned)slots, ctx->sm_count,
-                                           ctx->stream, &ws);
+                                           ctx->pool, ctx->stream, &ws);
     ctx->launches += ws.launches;
     if (e != cudaSuccess)
         return fail(ctx, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "%s: wavefront: %s", who,
@@ -846,7 +907,7 @@ int run_learned(mcrt_scene* sc, const TraceParams& P0, int sensor, const mcrt_tr
     unsigned* cnt = nullptr;
     cudaError_t e = cudaSuccess;
     auto A = [&](auto** p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(p), bytes ? bytes : 16, ctx->stream);
+        if (e == cudaSuccess) e = dalloc(ctx, p, bytes);
     };
     A(&qa, B * 64); A(&qb, B * 64); A(&fa, B * 32); A(&fb, B * 32); A(&mix, B * 192); A(&fin, B * 4);
     A(&cnt, 16);
@@ -983,6 +1044,7 @@ int run_learned(mcrt_scene* sc, const TraceParams& P0, int sensor, const mcrt_tr
     t->kernel_ms = ms;
     int terr = 0;
     CK(ctx, tc5_take_error(&terr, ctx->stream));
+    pool_trim(ctx->pool);
     if (terr) return fail(ctx, MCRT_ERR_TIMEOUT, "%s: a tensor-core wait of the proposal network ran out", who);
     if (status == 1) return fail(ctx, MCRT_ERR_TIMEOUT, "%s: deadline of %g ms expired", who, o->deadline_ms);
     if (status == 2) return fail(ctx, MCRT_ERR_CANCELLED, "%s: cancelled", who);
@@ -1242,8 +1304,7 @@ int batch_tally(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, mcrt_tal
     for (int i = 0; i < n; ++i) t->cell_n[i] = items[i].npaths;
     if (t->d_cell_n) dfree(ctx, t->d_cell_n);
     t->d_cell_n = nullptr;
-    CK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&t->d_cell_n), sizeof(unsigned long long) * (size_t)n,
-                            ctx->stream));
+    CK(ctx, dalloc(ctx, &t->d_cell_n, sizeof(unsigned long long) * (size_t)n));
     CK(ctx, cudaMemcpyAsync(t->d_cell_n, t->cell_n.data(), sizeof(unsigned long long) * (size_t)n,
                             cudaMemcpyHostToDevice, ctx->stream));
     return MCRT_OK;
@@ -1278,7 +1339,7 @@ int mcrt_trace_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, con
     if (rc) return rc;
     mcrt_tally* t = *tally;
     BatchItem* d_items = nullptr;
-    CK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_items), sizeof(BatchItem) * (size_t)n, ctx->stream));
+    CK(ctx, dalloc(ctx, &d_items, sizeof(BatchItem) * (size_t)n));
     cudaError_t e = cudaMemcpyAsync(d_items, h.data(), sizeof(BatchItem) * (size_t)n, cudaMemcpyHostToDevice,
                                     ctx->stream);
     TraceParams P = batch_params(h, d_items, total, o, t);
@@ -1619,6 +1680,7 @@ int mcrt_tally_destroy(mcrt_tally* t)
     dfree(ctx, t->d_out);
     dfree(ctx, t->d_cell_n);
     cudaStreamSynchronize(ctx->stream);
+    pool_trim(ctx->pool);
     delete t;
     return MCRT_OK;
 }
@@ -1672,8 +1734,7 @@ int mcrt_debug_pool_usage(mcrt_ctx* ctx, int32_t reset_high, uint64_t* used_curr
     if (!ctx || !used_current || !used_high) return fail(ctx, MCRT_ERR_ARG, "mcrt_debug_pool_usage: NULL argument");
     CK(ctx, cudaSetDevice(ctx->device));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
-    cudaMemPool_t pool;
-    CK(ctx, cudaDeviceGetMemPool(&pool, ctx->device));
+    const cudaMemPool_t pool = ctx->pool;
     unsigned long long cur = 0, high = 0;
     CK(ctx, cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &cur));
     CK(ctx, cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &high));
@@ -1751,7 +1812,7 @@ int mcrt_debug_terrain(const mcrt_scene* sc, int32_t n, const float* o, const fl
     if (n == 0) return MCRT_OK;
     CK(ctx, cudaSetDevice(ctx->device));
     float* buf = nullptr;
-    CK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&buf), (size_t)n * 7 * sizeof(float), ctx->stream));
+    CK(ctx, dalloc(ctx, &buf, (size_t)n * 7 * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(buf, o, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(buf + 3 * (size_t)n, d, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
@@ -1777,7 +1838,7 @@ int mcrt_debug_terrain_height(const mcrt_scene* sc, int32_t n, const float* xy, 
     if (n == 0) return MCRT_OK;
     CK(ctx, cudaSetDevice(ctx->device));
     float* buf = nullptr;
-    CK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&buf), (size_t)n * 6 * sizeof(float), ctx->stream));
+    CK(ctx, dalloc(ctx, &buf, (size_t)n * 6 * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(buf, xy, (size_t)n * 2 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) {
         ctx->launches++;

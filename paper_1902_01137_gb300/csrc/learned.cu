@@ -65,14 +65,13 @@ __global__ void f32_to_bf16_rows_kernel(const float* __restrict__ src, int n, in
 int alloc_proposal(mcrt_ctx* ctx, mcrt_proposal* P)
 {
     const size_t np = kMlpParams * sizeof(float);
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_params), np, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_m), np, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_v), np, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_grad), np, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_loss), sizeof(float), ctx->stream));
-    LCK(ctx, cudaMallocAsync(&P->d_wbf, mlp_packed_bf16_elems() * 2, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&P->d_bias), mlp_packed_bias_elems() * sizeof(float),
-                             ctx->stream));
+    LCK(ctx, pool_alloc(ctx, &P->d_params, np));
+    LCK(ctx, pool_alloc(ctx, &P->d_m, np));
+    LCK(ctx, pool_alloc(ctx, &P->d_v, np));
+    LCK(ctx, pool_alloc(ctx, &P->d_grad, np));
+    LCK(ctx, pool_alloc(ctx, &P->d_loss, sizeof(float)));
+    LCK(ctx, pool_alloc(ctx, &P->d_wbf, mlp_packed_bf16_elems() * 2));
+    LCK(ctx, pool_alloc(ctx, &P->d_bias, mlp_packed_bias_elems() * sizeof(float)));
     LCK(ctx, cudaMemsetAsync(P->d_m, 0, np, ctx->stream));
     LCK(ctx, cudaMemsetAsync(P->d_v, 0, np, ctx->stream));
     return MCRT_OK;
@@ -127,6 +126,7 @@ int mcrt_proposal_destroy(mcrt_proposal* P)
                     (void*)P->d_bias})
         if (p) cudaFreeAsync(p, ctx->stream);
     cudaStreamSynchronize(ctx->stream);
+    pool_trim(ctx->pool);
     delete P;
     return MCRT_OK;
 }
@@ -216,10 +216,10 @@ int mcrt_proposal_eval(mcrt_proposal* P, const float* host_feat, size_t n, float
     float* d_f32 = nullptr;
     void* d_feat = nullptr;
     float *d_mix = nullptr, *d_raw = nullptr;
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_f32), n * 9 * sizeof(float), ctx->stream));
-    LCK(ctx, cudaMallocAsync(&d_feat, n * 16 * 2, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_mix), n * 40 * sizeof(float), ctx->stream));
-    if (host_raw) LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_raw), n * 40 * sizeof(float), ctx->stream));
+    LCK(ctx, pool_alloc(ctx, &d_f32, n * 9 * sizeof(float)));
+    LCK(ctx, pool_alloc(ctx, &d_feat, n * 16 * 2));
+    LCK(ctx, pool_alloc(ctx, &d_mix, n * 40 * sizeof(float)));
+    if (host_raw) LCK(ctx, pool_alloc(ctx, &d_raw, n * 40 * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(d_f32, host_feat, n * 9 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) { ctx->launches++; e = launch_f32_to_bf16_rows(d_f32, (int)n, 9, d_feat, 16, ctx->stream); }
     if (e == cudaSuccess) {
@@ -253,10 +253,10 @@ int mcrt_proposal_train_step(mcrt_proposal* P, const float* host_feat, const flo
     LCK(ctx, cudaSetDevice(ctx->device));
     float *d_f32 = nullptr, *d_dirs = nullptr, *d_t = nullptr;
     void* d_feat = nullptr;
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_f32), n * 9 * sizeof(float), ctx->stream));
-    LCK(ctx, cudaMallocAsync(&d_feat, n * 16 * 2, ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_dirs), n * 3 * sizeof(float), ctx->stream));
-    LCK(ctx, cudaMallocAsync(reinterpret_cast<void**>(&d_t), n * sizeof(float), ctx->stream));
+    LCK(ctx, pool_alloc(ctx, &d_f32, n * 9 * sizeof(float)));
+    LCK(ctx, pool_alloc(ctx, &d_feat, n * 16 * 2));
+    LCK(ctx, pool_alloc(ctx, &d_dirs, n * 3 * sizeof(float)));
+    LCK(ctx, pool_alloc(ctx, &d_t, n * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(d_f32, host_feat, n * 9 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_dirs, host_dirs, n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_t, host_targets, n * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);

@@ -567,8 +567,8 @@ int wavefront_blocks_per_sm(bool bf16)
     return std::max(1, std::min(a, b));
 }
 
-cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, int sm_count, cudaStream_t st,
-                             WavefrontStats* stats)
+cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, int sm_count, cudaMemPool_t pool,
+                             cudaStream_t st, WavefrontStats* stats)
 {
     *stats = WavefrontStats{};
     const unsigned cap = slots;
@@ -577,7 +577,7 @@ cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, in
     W.cap = cap;
     char* buf = nullptr;
     const size_t qb = queue_bytes(cap);
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&buf), 3 * qb + 256, st);
+    cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&buf), 3 * qb + 256, pool, st);
     if (e != cudaSuccess) return e;
     carve(W.F[0], buf, cap);
     carve(W.F[1], buf + qb, cap);
