@@ -376,11 +376,10 @@ int mcrt_scene_build_majorants(mcrt_scene* sc, int32_t levels)
     }
     CK(ctx, cudaSetDevice(ctx->device));
     for (int L = 2; L <= levels; ++L) {
-        LAUNCH(ctx, launch_reduce_level(sc->d_pyr + sc->lev_off[L - 1], &sc->lev_dims[3 * (L - 1)],
-                                        sc->d_pyr + sc->lev_off[L], &sc->lev_dims[3 * L], false, ctx->stream));
         float* mn = sc->d_pyr + sc->pyr_capacity;
-        LAUNCH(ctx, launch_reduce_level(mn + sc->lev_off[L - 1], &sc->lev_dims[3 * (L - 1)], mn + sc->lev_off[L],
-                                        &sc->lev_dims[3 * L], true, ctx->stream));
+        LAUNCH(ctx, launch_reduce_level(sc->d_pyr + sc->lev_off[L - 1], mn + sc->lev_off[L - 1],
+                                        &sc->lev_dims[3 * (L - 1)], sc->d_pyr + sc->lev_off[L], mn + sc->lev_off[L],
+                                        &sc->lev_dims[3 * L], ctx->stream));
     }
     sc->levels = levels;
     sc->leaf_valid = false;
@@ -455,6 +454,7 @@ int mcrt_scene_build_octree(mcrt_scene* sc, int32_t levels)
         off[L] = tot;
         tot += (size_t)dims[3 * L] * dims[3 * L + 1] * dims[3 * L + 2];
     }
+    tot = (tot + 63) / 64 * 64;      // the min levels start on a vector boundary too
     const size_t n1 = (size_t)dims[3] * dims[4] * dims[5];
     // replace the previous octree (its leaf map goes with it)
     if (sc->leaf_grid == MCRT_GRID_OCTREE) sc->leaf_valid = false;
@@ -478,8 +478,8 @@ int mcrt_scene_build_octree(mcrt_scene* sc, int32_t levels)
     sc->oct_dims = dims;
     sc->oct_capacity = tot;
     sc->oct_levels = levels;
-    ctx->launches += (uint64_t)levels;
-    e = launch_octree(sc, make_dev_scene(sc, 0.0f), ctx->stream);
+    ctx->launches += (uint64_t)(levels > 3 ? levels - 2 : 1);
+    e = launch_octree(sc, ctx->stream);
     if (e != cudaSuccess) {
         sc->oct_levels = 0;
         return fail(ctx, MCRT_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
@@ -566,9 +566,10 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     // levels: 4 x 4 blocks while both sizes divide
     int lev = 1;
     while (lev < kMaxHfLevels && hnx % (1 << (2 * lev)) == 0 && hny % (1 << (2 * lev)) == 0) ++lev;
+    // (level 0 is stored only where it is the top one)
     int off[kMaxHfLevels] = {};
     size_t total = 0;
-    for (int L = 0; L < lev; ++L) {
+    for (int L = lev > 1 ? 1 : 0; L < lev; ++L) {
         off[L] = (int)total;
         total += (size_t)(hnx >> (2 * L)) * (size_t)(hny >> (2 * L));
     }
@@ -576,17 +577,21 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     float *dh = nullptr, *dp = nullptr;
     float4* dc = nullptr;
     int* bad = nullptr;
-    cudaError_t e = dalloc(ctx, &dh, n * sizeof(float));
-    if (e == cudaSuccess) e = dalloc(ctx, &dp, total * sizeof(float));
+    // heights on the device are read where they are (the call waits for the
+    // kernels below), host ones through a staging copy
+    const float* src = heights;
+    cudaError_t e = dalloc(ctx, &dp, total * sizeof(float));
     if (e == cudaSuccess) e = dalloc(ctx, &dc, n * sizeof(float4));
     if (e == cudaSuccess) e = dalloc(ctx, &bad, sizeof(int));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(dh, heights, n * sizeof(float),
-                            mem == MCRT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, ctx->stream);
+    if (e == cudaSuccess && mem == MCRT_MEM_HOST) {
+        e = dalloc(ctx, &dh, n * sizeof(float));
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dh, heights, n * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
+        src = dh;
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream);
     const float top = (float)sc->n[2] * sc->h[2];
-    if (e == cudaSuccess) { ctx->launches++; e = launch_hf_check(dh, (long long)n, top, bad, ctx->stream); }
-    if (e == cudaSuccess) { ctx->launches += lev; e = launch_hf_pyramid(dh, hnx, hny, dc, dp, off, lev, ctx->stream); }
+    if (e == cudaSuccess) { ctx->launches++; e = launch_hf_check(src, (long long)n, top, bad, ctx->stream); }
+    if (e == cudaSuccess) { ctx->launches += lev > 1 ? lev - 1 : 1; e = launch_hf_pyramid(src, hnx, hny, dc, dp, off, lev, ctx->stream); }
     const size_t ntop = (size_t)(hnx >> (2 * (lev - 1))) * (size_t)(hny >> (2 * (lev - 1)));
     std::vector<float> tops(ntop);
     int hbad = 0;
@@ -805,14 +810,23 @@ int make_claim_order(mcrt_scene* sc, const TraceParams& P, uint32_t** d_order, c
     return MCRT_OK;
 }
 
+// Launch shape of a plain trace: threads per block, and blocks.
+int trace_grid(mcrt_scene* sc, const TraceParams& P, int sensor, const mcrt_trace_opts* o, int* block)
+{
+    *block = o->block_size ? o->block_size : 128;
+    if (o->grid_size) return o->grid_size;
+    return sc->ctx->sm_count * trace_blocks_per_sm(sensor, sc->storage == MCRT_STORAGE_BF16, o->count_events != 0,
+                                                   P.S.hf != nullptr, o->sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh,
+                                                   *block);
+}
+
 int run_trace(mcrt_scene* sc, TraceParams& P, int sensor, const mcrt_trace_opts* o, mcrt_tally* t, const char* who)
 {
     mcrt_ctx* ctx = sc->ctx;
     const bool bf16 = sc->storage == MCRT_STORAGE_BF16;
     const bool count = o->count_events != 0;
-    const int block = o->block_size ? o->block_size : 128;
-    int grid = o->grid_size;
-    if (!grid) grid = ctx->sm_count * trace_blocks_per_sm(sensor, bf16, count, P.S.hf != nullptr, P.sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh, block);
+    int block = 0;
+    const int grid = trace_grid(sc, P, sensor, o, &block);
     if (!o->chunk) P.chunk = auto_chunk(P.total, ctx->sm_count, o->grid_size, block, sensor == kCamera ? P.spp : 0u);
     P.s1 = t->d_s1;
     P.s2 = t->d_s2;
@@ -1130,7 +1144,13 @@ int mcrt_trace_camera(mcrt_scene* sc, const mcrt_camera_desc* cam, uint32_t spp,
         return run_learned(sc, P, kCamera, o, t, spp, who);
     }
     uint32_t* d_order = nullptr;
-    if (o->pixel_order == MCRT_ORDER_COST) {
+    // (with a lane for every path all of them start at once: an order costs a
+    // walk of the view rays and two synchronisations, 0.3 ms, and changes
+    // nothing; a shard is defined by it)
+    int block = 0;
+    const bool all_at_once = o->schedule == MCRT_SCHEDULE_PERSISTENT && o->shard_count <= 1 &&
+                             P.total <= (unsigned long long)trace_grid(sc, P, kCamera, o, &block) * (unsigned)block;
+    if (o->pixel_order == MCRT_ORDER_COST && !all_at_once) {
         rc = make_claim_order(sc, P, &d_order, who);
         if (rc) return rc;
         P.pix_order = d_order;

@@ -258,10 +258,10 @@ enum Sensor { kCamera = 0, kFlux = 1 };
 
 // Launchers (return cudaError of the launch).
 cudaError_t launch_relayout(const float* src, const mcrt_scene* sc, cudaStream_t st);
-cudaError_t launch_reduce_level(const float* prev, const int* prev_dims, float* out, const int* dims, bool min_level,
-                                cudaStream_t st);
+cudaError_t launch_reduce_level(const float* pmax, const float* pmin, const int* prev_dims, float* omax, float* omin,
+                                const int* dims, cudaStream_t st);
 cudaError_t launch_leafmap(const mcrt_scene* sc, float tau, int finest, int grid, cudaStream_t st);
-cudaError_t launch_octree(const mcrt_scene* sc, const DevScene& S, cudaStream_t st);
+cudaError_t launch_octree(const mcrt_scene* sc, cudaStream_t st);
 cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float4* cells, float* pyr, const int* off, int levels,
                               cudaStream_t st);
 cudaError_t launch_hf_check(const float* h, long long n, float top, int* bad, cudaStream_t st);
