@@ -1445,7 +1445,7 @@ struct mcrt_batch_plan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    double* h_out = nullptr;       // pinned: (mean, se) per entry
+    double* h_out = nullptr;       // pinned: means, then standard errors
     WorkState* h_ws = nullptr;     // pinned: the kernel's status
 };
 
@@ -1596,10 +1596,8 @@ int mcrt_batch_plan_run(mcrt_batch_plan* p, double* mean, double* se, size_t cou
     p->t->kernel_ms = ms;
     if (kernel_ms) *kernel_ms = ms;
     if (p->h_ws->status != 0) return fail(ctx, MCRT_ERR_CUDA, "mcrt_batch_plan_run: kernel status %d", p->h_ws->status);
-    for (size_t i = 0; i < m; ++i) {
-        if (mean) mean[i] = p->h_out[2 * i];
-        if (se) se[i] = p->h_out[2 * i + 1];
-    }
+    if (mean) std::memcpy(mean, p->h_out, m * sizeof(double));
+    if (se) std::memcpy(se, p->h_out + m, m * sizeof(double));
     return MCRT_OK;
 }
 
@@ -1639,19 +1637,12 @@ int mcrt_tally_read(const mcrt_tally* t, double* mean, double* se, uint64_t* n, 
     if (mean || se) {
         LAUNCH(ctx, launch_finalize(t->d_s1, t->d_s2, (double)t->n_per_cell, (int)m,
                                     t->cell_n.empty() ? nullptr : t->d_cell_n, t->nq, t->d_out, ctx->stream));
-        double* h = new (std::nothrow) double[2 * m];
-        if (!h) return fail(ctx, MCRT_ERR_OOM, "mcrt_tally_read: host allocation failed");
-        cudaError_t e = cudaMemcpyAsync(h, t->d_out, 2 * m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+        cudaError_t e = cudaSuccess;
+        if (mean) e = cudaMemcpyAsync(mean, t->d_out, m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+        if (se && e == cudaSuccess)
+            e = cudaMemcpyAsync(se, t->d_out + m, m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) {
-            delete[] h;
-            return fail(ctx, MCRT_ERR_CUDA, "mcrt_tally_read: %s", cudaGetErrorString(e));
-        }
-        for (size_t i = 0; i < m; ++i) {
-            if (mean) mean[i] = h[2 * i];
-            if (se) se[i] = h[2 * i + 1];
-        }
-        delete[] h;
+        if (e != cudaSuccess) return fail(ctx, MCRT_ERR_CUDA, "mcrt_tally_read: %s", cudaGetErrorString(e));
     }
     if (n)
         for (size_t i = 0; i < m; ++i) n[i] = t->cell_n.empty() ? t->n_per_cell : t->cell_n[i / t->nq];

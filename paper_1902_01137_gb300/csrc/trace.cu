@@ -144,13 +144,17 @@ constexpr uint32_t kMaxHelpers = 5;
 // cycles per vertex with a helper, 8,000 without; 64 x 64 x 16 paths of the
 // blob field 2.5 -> 2.05 ms, a 500 x 301 x 16 image 10.5 -> 9.3 ms.
 
+// A batch's kernel holds its lane's scene pointer and derivative sums besides:
+// 12 fields 89.6 ms with spills at 8 blocks of 128, 88.0 without at 7.
+constexpr int kBatchBlocks = 7;
+
 // EXTRA: the variants that also handle decomposition tracking of sun rays
 // and Rayleigh clear air (chosen at run time); the others carry neither, so
 // the paper's estimator keeps its registers.  In batches, EXTRA instead
 // adds the dT/dalpha estimate.
 template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, bool BATCH = false, bool TERRAIN = false,
           bool EXTRA = false>
-__global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const __grid_constant__ TraceParams P)
+__global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLOCKS) trace_kernel(const __grid_constant__ TraceParams P)
 {
     // quantities per path: camera radiance; flux T_dir, T_dif, T_tot (+ dT/dg, dT/dalpha in batches)
     constexpr int NQ = (SENSOR == kCamera) ? 1 : (BATCH ? 5 : 3);
@@ -1143,8 +1147,9 @@ __global__ void __launch_bounds__(128, MCRT_TRACE_MIN_BLOCKS) trace_kernel(const
     }
 }
 
-// Mean and standard error of each tally entry from its FP64 sums; a batch
-// passes each cell's own path count (cell_n, nq entries per cell).
+// Mean and standard error of each tally entry from its FP64 sums, all means
+// first, so that each array goes to the caller's in one copy; a batch passes
+// each cell's own path count (cell_n, nq entries per cell).
 __global__ void finalize_kernel(const double* __restrict__ s1, const double* __restrict__ s2, double n_all, int count,
                                 const unsigned long long* __restrict__ cell_n, int nq, double* __restrict__ out)
 {
@@ -1154,8 +1159,8 @@ __global__ void finalize_kernel(const double* __restrict__ s1, const double* __r
     const double m = s1[i] / n;
     double var = s2[i] / n - m * m;
     if (var < 0.0) var = 0.0;
-    out[2 * i] = m;
-    out[2 * i + 1] = n > 1.0 ? sqrt(var / (n - 1.0)) : 0.0;
+    out[i] = m;
+    out[(size_t)count + i] = n > 1.0 ? sqrt(var / (n - 1.0)) : 0.0;
 }
 
 // One thread walks one ray and records its leaves (traversal check), with
