@@ -1139,7 +1139,7 @@ int mcrt_trace_camera(mcrt_scene* sc, const mcrt_camera_desc* cam, uint32_t spp,
         P.max_order = o->max_order;
         P.sun_mode = o->sun_mode;
         P.max_steps = 1u << 22;
-        set_rare_batch(P, o->rare_batch);
+        set_rare_batch(P, o->rare_batch, true);
         P.s1 = t->d_s1; P.s2 = t->d_s2; P.counters = t->d_counters; P.work = static_cast<WorkState*>(t->d_work);
         return run_learned(sc, P, kCamera, o, t, spp, who);
     }
@@ -1220,7 +1220,7 @@ int mcrt_trace_flux(mcrt_scene* sc, uint64_t npaths, uint64_t seed, const mcrt_t
         P.max_order = o->max_order;
         P.sun_mode = o->sun_mode;
         P.max_steps = 1u << 22;
-        set_rare_batch(P, o->rare_batch);
+        set_rare_batch(P, o->rare_batch, true);
         P.s1 = t->d_s1; P.s2 = t->d_s2; P.counters = t->d_counters; P.work = static_cast<WorkState*>(t->d_work);
         return run_learned(sc, P, kFlux, o, t, 1ull, who);
     }

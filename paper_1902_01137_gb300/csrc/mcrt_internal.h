@@ -228,12 +228,13 @@ struct TraceParams {
 // runs half empty: cumulus image of 16.8 M paths 62.1, 57.3, 56.3, 57.9,
 // 64.2 ms at 8, 12, 16, 20, 24 lanes; flux of the same field 53.3, 51.7,
 // 49.9, 48.3, 52.1 ms; octree image 35.2, 32.8, 32.3, 32.9, 35.3 ms.
-// Over a heightfield, where a pass costs more (and walkers wait besides): 20.0,
-// 19.6, 19.3, 19.2 ms at 16, 18, 20, 22.
-constexpr int kDefaultRareBatch = 16, kDefaultRareBatchHf = 20;
-inline void set_rare_batch(TraceParams& P, int requested)
+// Where a pass costs more it pays to wait longer: over a heightfield (walkers
+// wait besides) 20.0, 19.6, 19.3, 19.2 ms at 16, 18, 20, 22, in the learned
+// mode's passes 18.6, 18.5, 18.2 at 16, 18, 20.
+constexpr int kDefaultRareBatch = 16, kDefaultRareBatchLong = 20;
+inline void set_rare_batch(TraceParams& P, int requested, bool learned = false)
 {
-    P.rare_batch = requested > 0 ? requested : (P.S.hf ? kDefaultRareBatchHf : kDefaultRareBatch);
+    P.rare_batch = requested > 0 ? requested : (P.S.hf || learned ? kDefaultRareBatchLong : kDefaultRareBatch);
     P.min_steppers = 33 - P.rare_batch;
 }
 

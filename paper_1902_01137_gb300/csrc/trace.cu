@@ -156,6 +156,13 @@ template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, bool BATCH = false, b
           bool EXTRA = false>
 __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLOCKS) trace_kernel(const __grid_constant__ TraceParams P)
 {
+    // Steps between looks at who waits.  Two spare half of the votes and the
+    // loop: cumulus image of 16.8 M paths 49.5 -> 48.8 ms, 16.8 M flux paths 40.2
+    // -> 39.4, a 64 x 64 x 16 image 2.0 -> 1.75; three do not fit the instruction
+    // cache (52.9 ms), nor do two of the longer variants (4 M paths over a relief
+    // 19.2 -> 20.7, Rayleigh image 8.8 -> 9.3, batch 86.8 -> 87.7; with dT/dalpha,
+    // whose registers differ, 10.7 -> 10.4).
+    constexpr int kSteps = COUNT || TERRAIN || EXTRA != BATCH ? 1 : 2;
     // quantities per path: camera radiance; flux T_dir, T_dif, T_tot (+ dT/dg, dT/dalpha in batches)
     constexpr int NQ = (SENSOR == kCamera) ? 1 : (BATCH ? 5 : 3);
     // decomposition tracking needs the leaf minorants
@@ -993,117 +1000,120 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
         // ==== steps: until enough lanes wait for a rare pass ====================
         unsigned stepping;
         do {
-            // (heightfield: a flight whose current leaf reaches down into the relief
-            //  layer first finds its ground hit, in a rare pass)
-            if (TERRAIN && phase == PH_STEP && R.texit >= tpend) {
-                phase = PH_WALK;
-                tpend = kInf;
-            }
-            if (COUNT) {
-                const unsigned st = __ballot_sync(kFull, phase == PH_STEP), lv = __ballot_sync(kFull, phase != PH_IDLE);
-                occ[0] += 1; occ[1] += __popc(lv); occ[2] += __popc(st); occ[5] += __popc(lv) - __popc(st);
-                occ[7] += 32 - __popc(lv);
-                if (phase == PH_STEP) ++path_iters;
-            }
-            if (phase == PH_STEP) {
-                // one step: to the tentative collision inside the leaf, or across
-                // the leaf's exit face; both share the point and voxel arithmetic.
-                // Tracking majorant: the leaf's M, or M - m for a sun ray in
-                // decomposition tracking (the minorant m is applied exactly)
-                const bool decomp = DECOMP && kind != kMain && P.sun_mode == MCRT_SUN_DECOMP;
-                const float Mt = decomp ? R.M - R.mn : R.M;
-                const float te = TERRAIN ? fminf(R.texit, tg) : R.texit;
-                const float Mseg = Mt * (te - R.t);
-                const bool tent = Mt > 0.0f && tau < Mseg;
-                const bool at_ground = TERRAIN && !tent && tg <= R.texit;   // the surface cuts this leaf
-                const float tn = tent ? fminf(R.t + __fdividef(tau, Mt), te) : (at_ground ? tg : R.texit);
-                if (decomp) Ts *= __expf(-R.mn * (tn - R.t));   // the control over this piece of the leaf
-                float p[3];
-                int nv[3];
-                advance(Z, R, tn, !tent && !at_ground, p, nv);
-                const bool face = !tent && !at_ground;
-                int st = kInside;
-                uint2 e = make_uint2(0u, 0u);
-                if (face) {
-                    tau -= Mseg;
-                    float wdt;
-                    st = cross_face(Z, R, p, nv, &wdt);
-                    if (TERRAIN) { tg -= wdt; tpend -= wdt; }   // a periodic wrap restarts the segment
-                    if (st == kInside) e = __ldg(leaf_entry(Z, nv));
+#pragma unroll
+            for (int half = 0; half < kSteps; ++half) {
+                // (heightfield: a flight whose current leaf reaches down into the relief
+                //  layer first finds its ground hit, in a rare pass)
+                if (TERRAIN && phase == PH_STEP && R.texit >= tpend) {
+                    phase = PH_WALK;
+                    tpend = kInf;
                 }
-                if (tent) R.t = tn;
-                // the block of a tentative collision, or of the roulette at a leaf
-                // crossing of decomposition tracking (word 3, which uses it up)
-                const bool roulette = DECOMP && decomp && face && st == kInside && Ts < 0.1f;
-                const bool loads = tent && R.msk != 0;
-                if (COUNT && tent) {
-                    ++tents;
-                    if (kind == kMain) cnt[C_TENT]++;
-                    else cnt[C_SUN_TENT]++;
+                if (COUNT) {
+                    const unsigned st = __ballot_sync(kFull, phase == PH_STEP), lv = __ballot_sync(kFull, phase != PH_IDLE);
+                    occ[0] += 1; occ[1] += __popc(lv); occ[2] += __popc(st); occ[5] += __popc(lv) - __popc(st);
+                    occ[7] += 32 - __popc(lv);
+                    if (phase == PH_STEP) ++path_iters;
                 }
-                uint4 x = make_uint4(0u, 0u, 0u, 0u);
-                if (loads || roulette) {
-                    float k = 0.0f;
-                    if (!DECOMP || loads) {
-                        const size_t idx = brick_index(Z, nv[0], nv[1], nv[2]);
-                        k = BF16 ? __uint_as_float((uint32_t)__ldg(Z.vox16 + idx) << 16) : __ldg(Z.vox + idx);
-                        k = __fadd_rn(k, Z.k_gas);
+                if (phase == PH_STEP) {
+                    // one step: to the tentative collision inside the leaf, or across
+                    // the leaf's exit face; both share the point and voxel arithmetic.
+                    // Tracking majorant: the leaf's M, or M - m for a sun ray in
+                    // decomposition tracking (the minorant m is applied exactly)
+                    const bool decomp = DECOMP && kind != kMain && P.sun_mode == MCRT_SUN_DECOMP;
+                    const float Mt = decomp ? R.M - R.mn : R.M;
+                    const float te = TERRAIN ? fminf(R.texit, tg) : R.texit;
+                    const float Mseg = Mt * (te - R.t);
+                    const bool tent = Mt > 0.0f && tau < Mseg;
+                    const bool at_ground = TERRAIN && !tent && tg <= R.texit;   // the surface cuts this leaf
+                    const float tn = tent ? fminf(R.t + __fdividef(tau, Mt), te) : (at_ground ? tg : R.texit);
+                    if (decomp) Ts *= __expf(-R.mn * (tn - R.t));   // the control over this piece of the leaf
+                    float p[3];
+                    int nv[3];
+                    advance(Z, R, tn, !tent && !at_ground, p, nv);
+                    const bool face = !tent && !at_ground;
+                    int st = kInside;
+                    uint2 e = make_uint2(0u, 0u);
+                    if (face) {
+                        tau -= Mseg;
+                        float wdt;
+                        st = cross_face(Z, R, p, nv, &wdt);
+                        if (TERRAIN) { tg -= wdt; tpend -= wdt; }   // a periodic wrap restarts the segment
+                        if (st == kInside) e = __ldg(leaf_entry(Z, nv));
                     }
-                    const uint32_t ev = geti(K_EV) & ~kTermAfter;
-                    x = block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk);
-                    ++blk;
-                    if (!DECOMP || loads) {
-                        const float u0 = u01(x.x);
-                        if (kind == kMain) {
-                            if (u0 * R.M <= k) {
-                                F(K_VK) = k;
-                                phase = PH_REAL;
-                                if (LEARNED) { seti(K_NX, (uint32_t)nv[0]); seti(K_NY, (uint32_t)nv[1]); seti(K_NZ, (uint32_t)nv[2]); }
+                    if (tent) R.t = tn;
+                    // the block of a tentative collision, or of the roulette at a leaf
+                    // crossing of decomposition tracking (word 3, which uses it up)
+                    const bool roulette = DECOMP && decomp && face && st == kInside && Ts < 0.1f;
+                    const bool loads = tent && R.msk != 0;
+                    if (COUNT && tent) {
+                        ++tents;
+                        if (kind == kMain) cnt[C_TENT]++;
+                        else cnt[C_SUN_TENT]++;
+                    }
+                    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                    if (loads || roulette) {
+                        float k = 0.0f;
+                        if (!DECOMP || loads) {
+                            const size_t idx = brick_index(Z, nv[0], nv[1], nv[2]);
+                            k = BF16 ? __uint_as_float((uint32_t)__ldg(Z.vox16 + idx) << 16) : __ldg(Z.vox + idx);
+                            k = __fadd_rn(k, Z.k_gas);
+                        }
+                        const uint32_t ev = geti(K_EV) & ~kTermAfter;
+                        x = block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk);
+                        ++blk;
+                        if (!DECOMP || loads) {
+                            const float u0 = u01(x.x);
+                            if (kind == kMain) {
+                                if (u0 * R.M <= k) {
+                                    F(K_VK) = k;
+                                    phase = PH_REAL;
+                                    if (LEARNED) { seti(K_NX, (uint32_t)nv[0]); seti(K_NY, (uint32_t)nv[1]); seti(K_NZ, (uint32_t)nv[2]); }
+                                }
+                            } else if (P.sun_mode == MCRT_SUN_DELTA) {
+                                if (u0 * R.M <= k) { Ts = 0.0f; phase = PH_SUN_END; }
+                            } else {
+                                Ts *= decomp ? null_share<!EXTRA>(k - R.mn, R.M - R.mn) : null_share<!EXTRA>(k, R.M);
+                                if (!(Ts > 0.0f)) {
+                                    Ts = 0.0f;
+                                    phase = PH_SUN_END;
+                                } else if (Ts < 0.1f) {
+                                    if (u0 * 0.1f <= Ts) Ts = 0.1f;
+                                    else { Ts = 0.0f; phase = PH_SUN_END; }
+                                }
                             }
-                        } else if (P.sun_mode == MCRT_SUN_DELTA) {
-                            if (u0 * R.M <= k) { Ts = 0.0f; phase = PH_SUN_END; }
-                        } else {
-                            Ts *= decomp ? null_share<!EXTRA>(k - R.mn, R.M - R.mn) : null_share<!EXTRA>(k, R.M);
-                            if (!(Ts > 0.0f)) {
+                            tau = -__logf(u01(x.y));
+                        }
+                    }
+                    if (tent) {
+                        if (!loads) phase = PH_HIT;
+                    } else if (at_ground) {
+                        R.t = tg;
+                        phase = PH_LAND;
+                    } else if (st == kInside) {
+                        if (roulette) {
+                            if (u01(x.w) * 0.1f <= Ts) Ts = 0.1f;
+                            else { Ts = 0.0f; phase = PH_SUN_END; }
+                        }
+                        if (!roulette || phase == PH_STEP) {
+                            if (COUNT) {
+                                if (kind == kMain) cnt[C_LEAF]++;
+                                else cnt[C_SUN_LEAF]++;
+                            }
+                            finish_leaf<BF16>(Z, R, nv, e);
+                            if (R.steps > P.max_steps) {
+                                if (COUNT) cnt[C_ABORT]++;
                                 Ts = 0.0f;
-                                phase = PH_SUN_END;
-                            } else if (Ts < 0.1f) {
-                                if (u0 * 0.1f <= Ts) Ts = 0.1f;
-                                else { Ts = 0.0f; phase = PH_SUN_END; }
+                                phase = kind == kMain ? PH_END : PH_SUN_END;
                             }
                         }
-                        tau = -__logf(u01(x.y));
+                    } else if (kind != kMain) {
+                        if (st == kGround) Ts = 0.0f;
+                        phase = PH_SUN_END;
+                    } else if (st == kTop) {
+                        phase = PH_END;
+                    } else {
+                        phase = PH_FLOOR;
                     }
-                }
-                if (tent) {
-                    if (!loads) phase = PH_HIT;
-                } else if (at_ground) {
-                    R.t = tg;
-                    phase = PH_LAND;
-                } else if (st == kInside) {
-                    if (roulette) {
-                        if (u01(x.w) * 0.1f <= Ts) Ts = 0.1f;
-                        else { Ts = 0.0f; phase = PH_SUN_END; }
-                    }
-                    if (!roulette || phase == PH_STEP) {
-                        if (COUNT) {
-                            if (kind == kMain) cnt[C_LEAF]++;
-                            else cnt[C_SUN_LEAF]++;
-                        }
-                        finish_leaf<BF16>(Z, R, nv, e);
-                        if (R.steps > P.max_steps) {
-                            if (COUNT) cnt[C_ABORT]++;
-                            Ts = 0.0f;
-                            phase = kind == kMain ? PH_END : PH_SUN_END;
-                        }
-                    }
-                } else if (kind != kMain) {
-                    if (st == kGround) Ts = 0.0f;
-                    phase = PH_SUN_END;
-                } else if (st == kTop) {
-                    phase = PH_END;
-                } else {
-                    phase = PH_FLOOR;
                 }
             }
             stepping = __ballot_sync(kFull, phase == PH_STEP);
