@@ -10,7 +10,11 @@
 // BF16 in the no-swizzle core-matrix layout of tc5.cuh, accumulation FP32.
 //
 //  * mlp_infer_tc5_kernel -- forward pass; the epilogue turns the 40 outputs
-//    of a row into unit lobe axes, concentrations and softmax weights.
+//    of a row into unit lobe axes, concentrations and softmax weights.  The
+//    epilogues' instructions bound it, not the products: with two floats per
+//    instruction, 16-byte staging and 4 CTAs per SM (one activation buffer
+//    instead of two) the eight passes of a 512 x 512 x 16 learned image take
+//    237, 191, 165, 141, 123, 106, 91 and 79 us, 390 to 120 before.
 //  * mlp_train_tc5_kernel -- forward, gradient of the KL loss with respect
 //    to the 40 outputs (FP32, CUDA cores), and the backward pass:
 //      dA_{l-1} = dZ_l W_l          M = 128 rows, N = 64, from TMEM
@@ -65,26 +69,81 @@ constexpr float kGeluC = 0.7978845608028654f;                 // sqrt(2 / pi)
 constexpr float kGeluAC = 0.044715f * 0.7978845608028654f;      // a c
 constexpr float kGelu3AC = 3.0f * 0.044715f * 0.7978845608028654f;
 
-__device__ __forceinline__ void gelu2(float x, float& h, float& gp)
+// Two floats per instruction (add, mul and fma .f32x2 of sm_100 and later,
+// each half rounded as the scalar operation): the epilogues below issue about
+// half as many FP32 instructions with them.
+struct F2 { unsigned long long v; };
+__device__ __forceinline__ F2 f2(float a, float b)
 {
-    const float x2 = x * x;
-    const float t = tanh_fast(x * fmaf(kGeluAC, x2, kGeluC));
-    const float hx = 0.5f * x;
-    h = fmaf(hx, t, hx);
-    gp = fmaf(hx * fmaf(-t, t, 1.0f), fmaf(kGelu3AC, x2, kGeluC), fmaf(0.5f, t, 0.5f));
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack(F2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 tanh2(F2 x)
+{
+    float a, b;
+    unpack(x, a, b);
+    return f2(tanh_fast(a), tanh_fast(b));
 }
 
-__device__ __forceinline__ float gelu1(float x)
+// GELU and its derivative of a pair.
+__device__ __forceinline__ void gelu2(F2 x, F2& h, F2& gp)
 {
-    const float t = tanh_fast(x * fmaf(kGeluAC, x * x, kGeluC));
-    const float hx = 0.5f * x;
-    return fmaf(hx, t, hx);
+    const F2 half = f2(0.5f, 0.5f);
+    const F2 x2 = mul2(x, x);
+    const F2 t = tanh2(mul2(x, fma2(f2(kGeluAC, kGeluAC), x2, f2(kGeluC, kGeluC))));
+    const F2 hx = mul2(half, x);
+    h = fma2(hx, t, hx);
+    const F2 nt = mul2(f2(-1.0f, -1.0f), t);
+    gp = fma2(mul2(hx, fma2(nt, t, f2(1.0f, 1.0f))), fma2(f2(kGelu3AC, kGelu3AC), x2, f2(kGeluC, kGeluC)),
+              fma2(half, t, half));
+}
+
+// GELU of a pair.
+__device__ __forceinline__ F2 gelu1(F2 x)
+{
+    const F2 t = tanh2(mul2(x, fma2(f2(kGeluAC, kGeluAC), mul2(x, x), f2(kGeluC, kGeluC))));
+    const F2 hx = mul2(f2(0.5f, 0.5f), x);
+    return fma2(hx, t, hx);
 }
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+__device__ __forceinline__ uint32_t pack2(F2 x)
+{
+    float a, b;
+    unpack(x, a, b);
+    return pack2(a, b);
+}
+
+// Bias pair c of a layer (even c; the bias block lies on 16 bytes).
+__device__ __forceinline__ F2 bias2(const float* b, int c)
+{
+    const float2 v = *reinterpret_cast<const float2*>(b + c);
+    return f2(v.x, v.y);
 }
 
 __device__ __forceinline__ void st16(uint8_t* base, uint32_t off, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
@@ -141,7 +200,8 @@ __device__ __forceinline__ bool from_mma(uint64_t* bar, uint32_t& phase)
 // exponential per lobe.
 constexpr int kTracerMix = 48;
 
-__device__ __forceinline__ void mixture_out(const float* r, float* __restrict__ o, bool tracer)
+template <bool TRACER>
+__device__ __forceinline__ void mixture_out(const float* r, float* o)
 {
     float mx = -3.0e38f;
 #pragma unroll
@@ -159,12 +219,12 @@ __device__ __forceinline__ void mixture_out(const float* r, float* __restrict__ 
         const float k = r[5 * j + 3];
         const float kap = (k > 20.0f ? k : log1pf(__expf(k))) + 1e-3f;
         const float pi = e[j] * inv_s;
-        const int b = tracer ? 6 * j : 5 * j;
+        const int b = TRACER ? 6 * j : 5 * j;
         o[b] = nn > 1e-24f ? x * inv : 0.0f;
         o[b + 1] = nn > 1e-24f ? y * inv : 0.0f;
         o[b + 2] = nn > 1e-24f ? z * inv : 1.0f;
         o[b + 3] = kap;
-        if (tracer) {
+        if (TRACER) {
             cdf += pi;
             o[b + 4] = cdf;
             o[b + 5] = pi * kap / (2.0f * kPi * (-expm1f(-2.0f * kap)));
@@ -177,10 +237,16 @@ __device__ __forceinline__ void mixture_out(const float* r, float* __restrict__ 
 // ---------------------------------------------------------------------------
 // Inference
 // ---------------------------------------------------------------------------
-constexpr uint32_t kInfOffHa = kOffSX + kSzX, kInfOffHb = kInfOffHa + kRows * 64 * 2;
-constexpr uint32_t kInfSmem = kInfOffHb + kRows * 64 * 2;          // 61,440 bytes
+// One activation buffer serves all layers (a layer's product has been read
+// when its epilogue writes the next operands); the output rows are staged
+// over it and the feature buffer, 52 words apart (16-byte accesses of eight
+// rows then touch every bank once).  51,200 bytes: 4 CTAs per SM.
+constexpr uint32_t kInfOffH = kOffSX + kSzX;
+constexpr int kStageLd = 52;
+constexpr uint32_t kInfSmem = kOffSX + kRows * kStageLd * 4;
 constexpr uint32_t kInfCols = 64;
-static_assert(kRows * (48 + 1) * 4 <= kInfSmem - kInfOffHa, "output staging fits in the two activation buffers");
+constexpr int kInfCtas = 4;
+static_assert(kInfOffH + kRows * 64 * 2 <= kInfSmem, "the activation buffer fits");
 
 // One forward epilogue: bias + GELU of the 64 accumulator columns, BF16 to
 // the next layer's operand rows.
@@ -194,24 +260,23 @@ __device__ __forceinline__ void infer_hidden(uint32_t tacc, const float* __restr
         uint32_t p[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-            p[j] = pack2(gelu1(__uint_as_float(v[2 * j]) + bias[c0 + 2 * j]),
-                         gelu1(__uint_as_float(v[2 * j + 1]) + bias[c0 + 2 * j + 1]));
+            p[j] = pack2(gelu1(add2(f2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), bias2(bias, c0 + 2 * j))));
         st16(H, core_off(row, c0, 64), p[0], p[1], p[2], p[3]);
         st16(H, core_off(row, c0 + 8, 64), p[4], p[5], p[6], p[7]);
     }
 }
 
-__global__ void __launch_bounds__(128) mlp_infer_tc5_kernel(const __nv_bfloat16* __restrict__ wpacked,
+template <bool TRACER>
+__global__ void __launch_bounds__(128, kInfCtas) mlp_infer_tc5_kernel(const __nv_bfloat16* __restrict__ wpacked,
                                                            const float* __restrict__ bpacked,
                                                            const __nv_bfloat16* __restrict__ feat, int n,
-                                                           float* __restrict__ mix, float* __restrict__ raw_out,
-                                                           int tracer_layout)
+                                                           float* __restrict__ mix, float* __restrict__ raw_out)
 {
     extern __shared__ __align__(1024) uint8_t sm[];
-    __shared__ float sB[kPackedBias];
+    __shared__ __align__(16) float sB[kPackedBias];
     __shared__ uint64_t bar;
     __shared__ uint32_t tbase;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     stage_weights(sm, wpacked, tid, 128);
     for (int i = tid; i < kPackedBias; i += 128) sB[i] = bpacked[i];
     if (tid == 0) { mbar_init(&bar, 1); fence_mbar_init(); }
@@ -221,7 +286,7 @@ __global__ void __launch_bounds__(128) mlp_infer_tc5_kernel(const __nv_bfloat16*
     const uint32_t tacc = T + ((uint32_t)(32 * warp) << 16);
     const uint32_t aW1 = smem_addr(sm + kOffSW1), aW2 = smem_addr(sm + kOffSW2), aW3 = smem_addr(sm + kOffSW3);
     const uint32_t aW4 = smem_addr(sm + kOffSW4), aX = smem_addr(sm + kOffSX);
-    const uint32_t aHa = smem_addr(sm + kInfOffHa), aHb = smem_addr(sm + kInfOffHb);
+    const uint32_t aH = smem_addr(sm + kInfOffH);
     constexpr uint32_t id64 = idesc_bf16(128, 64, false, false), id48 = idesc_bf16(128, 48, false, false);
     uint32_t phase = 0;
     bool ok = true;
@@ -243,27 +308,27 @@ __global__ void __launch_bounds__(128) mlp_infer_tc5_kernel(const __nv_bfloat16*
             mma_commit(&bar);
         }
         if (!(ok = from_mma(&bar, phase))) break;
-        infer_hidden(tacc, sB, sm + kInfOffHa, tid);
-        // layers 2 and 3: K = 64 in four steps, operands alternating between Ha and Hb
+        infer_hidden(tacc, sB, sm + kInfOffH, tid);
+        // layers 2 and 3: K = 64 in four steps
         for (int L = 0; L < 2 && ok; ++L) {
-            const uint32_t aIn = L == 0 ? aHa : aHb, aWl = L == 0 ? aW2 : aW3;
+            const uint32_t aWl = L == 0 ? aW2 : aW3;
             to_mma();
             if (tid == 0) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    mma_bf16(T, sdesc_kmajor(aIn + 256u * k, 64), sdesc_kmajor(aWl + 256u * k, 64), id64, k ? 1u : 0u);
+                    mma_bf16(T, sdesc_kmajor(aH + 256u * k, 64), sdesc_kmajor(aWl + 256u * k, 64), id64, k ? 1u : 0u);
                 mma_commit(&bar);
             }
             if (!(ok = from_mma(&bar, phase))) break;
-            infer_hidden(tacc, sB + 64 * (L + 1), sm + (L == 0 ? kInfOffHb : kInfOffHa), tid);
+            infer_hidden(tacc, sB + 64 * (L + 1), sm + kInfOffH, tid);
         }
         if (!ok) break;
-        // layer 4: Ha (K = 64) -> 48 output columns (40 used)
+        // layer 4: K = 64 -> 48 output columns (40 used)
         to_mma();
         if (tid == 0) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                mma_bf16(T, sdesc_kmajor(aHa + 256u * k, 64), sdesc_kmajor(aW4 + 256u * k, 64), id48, k ? 1u : 0u);
+                mma_bf16(T, sdesc_kmajor(aH + 256u * k, 64), sdesc_kmajor(aW4 + 256u * k, 64), id48, k ? 1u : 0u);
             mma_commit(&bar);
         }
         if (!(ok = from_mma(&bar, phase))) break;
@@ -276,21 +341,24 @@ __global__ void __launch_bounds__(128) mlp_infer_tc5_kernel(const __nv_bfloat16*
 #pragma unroll
             for (int j = 0; j < 16; ++j) r[c0 + j] = __uint_as_float(v[j]) + sB[192 + c0 + j];
         }
-        // the rows' mixtures go through shared memory (the activation
-        // buffers are free once layer 4 has run; stride W + 1 words: no bank
-        // conflicts) and out with a warp per row, so the stores coalesce
-        const int W = tracer_layout ? kTracerMix : kOut;
-        float* stage = reinterpret_cast<float*>(sm + kInfOffHa);
+        // the rows' mixtures go through shared memory (free once layer 4 has
+        // run), 16 bytes at a time, and out row after row, so the stores coalesce
+        constexpr int W4 = (TRACER ? kTracerMix : kOut) / 4;
+        float4* stage = reinterpret_cast<float4*>(sm + kOffSX);
         if (row < n) {
             if (raw_out)
                 for (int i = 0; i < kOut; ++i) raw_out[(size_t)row * kOut + i] = r[i];
-            mixture_out(r, stage + tid * (W + 1), tracer_layout != 0);
+            float o[4 * W4];
+            mixture_out<TRACER>(r, o);
+#pragma unroll
+            for (int c = 0; c < W4; ++c)
+                stage[tid * (kStageLd / 4) + c] = make_float4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
         }
         __syncthreads();
         const int nrows = min(kRows, n - tile * kRows);
-        for (int rr = warp; rr < nrows; rr += 4)
-            for (int c = lane; c < W; c += 32)
-                mix[(size_t)(tile * kRows + rr) * W + c] = stage[rr * (W + 1) + c];
+        float4* out = reinterpret_cast<float4*>(mix) + (size_t)tile * kRows * W4;
+        for (int q = tid; q < nrows * W4; q += 128) out[q] = stage[(q / W4) * (kStageLd / 4) + q % W4];
+        __syncthreads();
     }
     if (!ok && tid == 0) atomicExch(&g_tc5_error, 1);
     fence_before_sync();
@@ -323,10 +391,11 @@ __device__ __forceinline__ void train_hidden(uint32_t tl, uint32_t cgp, int c1, 
     uint32_t p[16], g[32];
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-        float h0, h1, g0, g1;
-        gelu2(__uint_as_float(v[2 * j]) + bias[c1 + 2 * j], h0, g0);
-        gelu2(__uint_as_float(v[2 * j + 1]) + bias[c1 + 2 * j + 1], h1, g1);
-        p[j] = pack2(h0, h1);
+        F2 h, gp;
+        float g0, g1;
+        gelu2(add2(f2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), bias2(bias, c1 + 2 * j)), h, gp);
+        unpack(gp, g0, g1);
+        p[j] = pack2(h);
         g[2 * j] = __float_as_uint(g0);
         g[2 * j + 1] = __float_as_uint(g1);
     }
@@ -348,8 +417,8 @@ __device__ __forceinline__ void train_dz(uint32_t tl, uint32_t cgp, int c1, uint
     uint32_t p[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-        p[j] = pack2(__uint_as_float(a[2 * j]) * __uint_as_float(g[2 * j]),
-                     __uint_as_float(a[2 * j + 1]) * __uint_as_float(g[2 * j + 1]));
+        p[j] = pack2(mul2(f2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])),
+                          f2(__uint_as_float(g[2 * j]), __uint_as_float(g[2 * j + 1]))));
 #pragma unroll
     for (int q = 0; q < 4; ++q) st16(DZ, core_off(row, c1 + 8 * q, kCD), p[4 * q], p[4 * q + 1], p[4 * q + 2], p[4 * q + 3]);
 }
@@ -461,7 +530,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) mlp_train_tc5_kernel(const __nv
                                                                      float* __restrict__ loss_out)
 {
     extern __shared__ __align__(1024) uint8_t sm[];
-    __shared__ float sB[kPackedBias];
+    __shared__ __align__(16) float sB[kPackedBias];
     __shared__ float xch[3][2][kRows];
     __shared__ uint64_t bar;
     __shared__ uint32_t tbase;
@@ -632,14 +701,13 @@ cudaError_t launch_mlp_infer(const void* wpacked, const float* bpacked, const vo
                              float* raw, int sm_count, cudaStream_t st, bool tracer_layout)
 {
     if (n <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(mlp_infer_tc5_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kInfSmem);
+    const auto kernel = tracer_layout ? mlp_infer_tc5_kernel<true> : mlp_infer_tc5_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInfSmem);
     if (e != cudaSuccess) return e;
     const int tiles = (n + kRows - 1) / kRows;
-    const int grid = tiles < 3 * sm_count ? tiles : 3 * sm_count;
-    mlp_infer_tc5_kernel<<<grid, 128, kInfSmem, st>>>(static_cast<const __nv_bfloat16*>(wpacked), bpacked,
-                                                      static_cast<const __nv_bfloat16*>(feat), n, mix, raw,
-                                                      tracer_layout ? 1 : 0);
+    const int grid = tiles < kInfCtas * sm_count ? tiles : kInfCtas * sm_count;
+    kernel<<<grid, 128, kInfSmem, st>>>(static_cast<const __nv_bfloat16*>(wpacked), bpacked,
+                                        static_cast<const __nv_bfloat16*>(feat), n, mix, raw);
     return cudaGetLastError();
 }
 
