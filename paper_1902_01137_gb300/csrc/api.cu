@@ -768,38 +768,44 @@ int make_claim_order(mcrt_scene* sc, const TraceParams& P, uint32_t** d_order, c
     int tx = 0;
     const int n = order_tiles(P.width, P.height, &tx);
     float* d_cost = nullptr;
-    uint32_t* d_tiles = nullptr;
-    CK(ctx, dalloc(ctx, &d_cost, (size_t)n * sizeof(float)));
-    ctx->launches++;
-    cudaError_t e = launch_view_cost(P, sc->storage == MCRT_STORAGE_BF16, d_cost, ctx->stream);
-    std::vector<float> cost((size_t)n);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(cost.data(), d_cost, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost,
-                                              ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    dfree(ctx, d_cost);
-    if (e != cudaSuccess) return fail(ctx, MCRT_ERR_CUDA, "%s: claim order: %s", who, cudaGetErrorString(e));
-    std::vector<uint32_t> tiles((size_t)2 * n);
-    for (int i = 0; i < n; ++i) {
-        tiles[i] = (uint32_t)i;
-        if (!(cost[i] >= 0.0f)) cost[i] = 3.0e38f;     // NaN: treat as the most costly
-    }
-    std::stable_sort(tiles.begin(), tiles.begin() + n, [&](uint32_t a, uint32_t b) { return cost[a] > cost[b]; });
-    uint32_t acc = 0;
-    for (int b = 0; b < n; ++b) {
-        const int x0 = (int)(tiles[b] % (uint32_t)tx) * 8, y0 = (int)(tiles[b] / (uint32_t)tx) * 8;
-        tiles[n + b] = acc;
-        acc += (uint32_t)(std::min(8, P.width - x0) * std::min(8, P.height - y0));
-    }
-    e = dalloc(ctx, &d_tiles, (size_t)2 * n * sizeof(uint32_t));
+    uint32_t* d_tiles = nullptr;      // the tiles in order, then the pixels before each
+    cudaError_t e = dalloc(ctx, &d_cost, (size_t)n * sizeof(float));
+    if (e == cudaSuccess) e = dalloc(ctx, &d_tiles, (size_t)2 * n * sizeof(uint32_t));
     if (e == cudaSuccess) e = dalloc(ctx, d_order, (size_t)P.width * P.height * sizeof(uint32_t));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_tiles, tiles.data(), (size_t)2 * n * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                            ctx->stream);
+    if (e == cudaSuccess) {
+        ctx->launches++;
+        e = launch_view_cost(P, sc->storage == MCRT_STORAGE_BF16, d_cost, ctx->stream);
+    }
+    if (e == cudaSuccess && sorts_on_device(n)) {
+        ctx->launches++;
+        e = launch_sort_tiles(d_cost, n, P.width, P.height, d_tiles, d_tiles + n, ctx->stream);
+    } else if (e == cudaSuccess) {
+        // more tiles than one block sorts: on the host
+        std::vector<float> cost((size_t)n);
+        e = cudaMemcpyAsync(cost.data(), d_cost, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        std::vector<uint32_t> tiles((size_t)2 * n);
+        for (int i = 0; i < n; ++i) {
+            tiles[i] = (uint32_t)i;
+            if (!(cost[i] >= 0.0f)) cost[i] = 3.0e38f;     // NaN: treat as the most costly
+        }
+        std::stable_sort(tiles.begin(), tiles.begin() + n, [&](uint32_t a, uint32_t b) { return cost[a] > cost[b]; });
+        uint32_t acc = 0;
+        for (int b = 0; b < n; ++b) {
+            const int x0 = (int)(tiles[b] % (uint32_t)tx) * 8, y0 = (int)(tiles[b] / (uint32_t)tx) * 8;
+            tiles[n + b] = acc;
+            acc += (uint32_t)(std::min(8, P.width - x0) * std::min(8, P.height - y0));
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d_tiles, tiles.data(), (size_t)2 * n * sizeof(uint32_t), cudaMemcpyHostToDevice,
+                                ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);    // the host vector is read by the copy
+    }
     if (e == cudaSuccess) {
         ctx->launches++;
         e = launch_expand_order(d_tiles, d_tiles + n, n, P.width, P.height, *d_order, ctx->stream);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);    // the host vector is read by the copy
+    dfree(ctx, d_cost);
     dfree(ctx, d_tiles);
     if (e != cudaSuccess) {
         dfree(ctx, *d_order);
@@ -1145,8 +1151,8 @@ int mcrt_trace_camera(mcrt_scene* sc, const mcrt_camera_desc* cam, uint32_t spp,
     }
     uint32_t* d_order = nullptr;
     // (with a lane for every path all of them start at once: an order costs a
-    // walk of the view rays and two synchronisations, 0.3 ms, and changes
-    // nothing; a shard is defined by it)
+    // walk of the view rays, a sort and their launches and changes nothing; a
+    // shard is defined by it)
     int block = 0;
     const bool all_at_once = o->schedule == MCRT_SCHEDULE_PERSISTENT && o->shard_count <= 1 &&
                              P.total <= (unsigned long long)trace_grid(sc, P, kCamera, o, &block) * (unsigned)block;

@@ -469,10 +469,9 @@ cudaError_t launch_octree(const mcrt_scene* sc, cudaStream_t st)
 
 // ---------------------------------------------------------------------------
 // Heightfield ground: max pyramid.  Level 0 holds each cell's maximum over
-// its 4 corner heights (periodic), which are kept as one record per cell;
-// level L the maximum over 4 x 4 cells of
-// level L - 1.  Also a scan for invalid heights (not finite, < 0 or above
-// the top of the field).
+// its 4 corner heights (periodic), which are kept as one record per cell,
+// level L the maximum over 4 x 4 cells of level L - 1.  Also a scan for
+// invalid heights (not finite, < 0 or above the top of the field).
 // ---------------------------------------------------------------------------
 namespace {
 

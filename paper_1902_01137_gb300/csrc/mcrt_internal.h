@@ -307,6 +307,9 @@ bool bounds_checked_build();
 cudaError_t read_bounds_violations(unsigned* count, unsigned* first_code);
 int order_tiles(int width, int height, int* tiles_x);
 cudaError_t launch_view_cost(const TraceParams& P, bool bf16, float* cost, cudaStream_t st);
+bool sorts_on_device(int n);
+cudaError_t launch_sort_tiles(const float* cost, int n, int width, int height, uint32_t* tiles, uint32_t* prefix,
+                              cudaStream_t st);
 cudaError_t launch_expand_order(const uint32_t* tiles, const uint32_t* prefix, int n, int width, int height,
                                 uint32_t* order, cudaStream_t st);
 cudaError_t launch_shard_order(const uint32_t* order, uint32_t n_out, uint32_t stride, uint32_t offset,

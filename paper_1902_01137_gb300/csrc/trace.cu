@@ -1266,6 +1266,76 @@ __global__ void view_cost_kernel(TraceParams P, int tiles_x, int tiles_y, float*
     cost[i] = c;
 }
 
+// Tiles by cost, largest first, ties in raster order (a NaN cost counts as the
+// largest), and the pixels before each: one block sorts up to kSortTiles keys
+// in shared memory by a bitonic network, ~cost bits above the tile's index.
+// One block, so bound by its 105 barriers at 16,384 tiles (a 1024 x 1024
+// image), which is what 128 KB of keys hold; larger images sort on the host,
+// where the copies and two waits cost more the smaller the trace is: a
+// 1023 x 767 x 15 octree image took 30.44 ms that way and 30.02 ms this way,
+// a 500 x 301 x 16 one 10.36 and 10.29.
+constexpr int kSortTiles = 16384;
+
+__global__ void __launch_bounds__(1024) sort_tiles_kernel(const float* __restrict__ cost, int n, int n2, int tiles_x,
+                                                          int width, int height, uint32_t* __restrict__ tiles,
+                                                          uint32_t* __restrict__ prefix)
+{
+    extern __shared__ unsigned long long key[];
+    __shared__ uint32_t warp_sum[32];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < n2; i += 1024) {
+        unsigned long long k = ~0ull;                      // padding: last
+        if (i < n) {
+            const float c = cost[i];
+            const float v = c > 0.0f ? c : c == 0.0f ? 0.0f : 3.0e38f;      // (-0 sorts as 0)
+            k = ((unsigned long long)~__float_as_uint(v) << 32) | (uint32_t)i;
+        }
+        key[i] = k;
+    }
+    __syncthreads();
+    for (int size = 2; size <= n2; size <<= 1)
+        for (int d = size >> 1; d > 0; d >>= 1) {
+            for (int q = tid; q < n2 / 2; q += 1024) {
+                const int a = 2 * q - (q & (d - 1)), b = a + d;
+                const unsigned long long x = key[a], y = key[b];
+                if ((x > y) == ((a & size) == 0)) {
+                    key[a] = y;
+                    key[b] = x;
+                }
+            }
+            __syncthreads();
+        }
+    // pixels before each tile: an exclusive scan, 1024 tiles at a time
+    uint32_t base = 0;
+    for (int i0 = 0; i0 < n; i0 += 1024) {
+        const int i = i0 + tid;
+        uint32_t tile = 0, px = 0;
+        if (i < n) {
+            tile = (uint32_t)key[i];
+            const int x0 = (int)(tile % (uint32_t)tiles_x) * kOrderTile, y0 = (int)(tile / (uint32_t)tiles_x) * kOrderTile;
+            px = (uint32_t)(min(kOrderTile, width - x0) * min(kOrderTile, height - y0));
+        }
+        uint32_t incl = px;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(kFull, incl, o);
+            if ((tid & 31) >= o) incl += v;
+        }
+        if ((tid & 31) == 31) warp_sum[tid >> 5] = incl;
+        __syncthreads();
+        uint32_t before = base, all = base;
+        for (int w = 0; w < 32; ++w) {
+            if (w < (tid >> 5)) before += warp_sum[w];
+            all += warp_sum[w];
+        }
+        if (i < n) {
+            tiles[i] = tile;
+            prefix[i] = before + incl - px;
+        }
+        base = all;
+        __syncthreads();
+    }
+}
+
 // order[prefix[b] + j] = the j-th pixel (row-major inside the tile) of the
 // b-th tile in claim order.
 // One shard of a claim order: out[i] = order[i * stride + offset] (the
@@ -1503,6 +1573,22 @@ cudaError_t launch_view_cost(const TraceParams& P, bool bf16, float* cost, cudaS
     const int ty = n / tx;
     if (bf16) view_cost_kernel<true><<<(n + 127) / 128, 128, 0, st>>>(P, tx, ty, cost);
     else view_cost_kernel<false><<<(n + 127) / 128, 128, 0, st>>>(P, tx, ty, cost);
+    return cudaGetLastError();
+}
+
+bool sorts_on_device(int n) { return n <= kSortTiles; }
+
+cudaError_t launch_sort_tiles(const float* cost, int n, int width, int height, uint32_t* tiles, uint32_t* prefix,
+                              cudaStream_t st)
+{
+    int tx = 0, n2 = 2;
+    order_tiles(width, height, &tx);
+    while (n2 < n) n2 <<= 1;
+    const size_t smem = (size_t)n2 * sizeof(unsigned long long);
+    cudaError_t e = cudaFuncSetAttribute(sort_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kSortTiles * (int)sizeof(unsigned long long));
+    if (e != cudaSuccess) return e;
+    sort_tiles_kernel<<<1, 1024, smem, st>>>(cost, n, n2, tx, width, height, tiles, prefix);
     return cudaGetLastError();
 }
 

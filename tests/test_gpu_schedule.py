@@ -65,3 +65,15 @@ def test_helped_batch_items_are_the_same(env, dalpha):
     items = [(flat, 0.0, 30.0, 0.0, 33, 1), (flat, 0.2, 70.0, 40.0, 2001, 2), (flat, 0.01, 10.0, 0.0, 1, 3)]
     _same(m.trace_batch(ctx, items, chunk=1, batch_dalpha=dalpha),
           m.trace_batch(ctx, items, chunk=1, grid_size=1, block_size=32, batch_dalpha=dalpha))
+
+
+@pytest.mark.parametrize("size", [(8, 8), (9, 7), (37, 21), (1000, 8), (8200, 3), (1024, 1024), (1025, 1024)])
+def test_claim_order_covers_the_image(env, size):
+    # 1, 2 (one ragged), 15, 125, 1025 and 16,384 tiles are sorted on the device, more on the host;
+    # a pixel left out or taken twice would change its sum
+    m, ctx, sp, flat, hilly = env
+    cam = scenes.nadir_camera(sp, *size)
+    kw = dict(seed=7, chunk=1) if size[0] * size[1] > 200000 else dict(seed=7, chunk=1, grid_size=1, block_size=32)
+    a = flat.trace_camera(cam, 1, pixel_order=m.MCRT_ORDER_COST, **kw)
+    b = flat.trace_camera(cam, 1, pixel_order=m.MCRT_ORDER_RASTER, **kw)
+    np.testing.assert_array_equal(a.mean, b.mean)
