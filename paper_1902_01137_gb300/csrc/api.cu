@@ -577,15 +577,23 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     float *dh = nullptr, *dp = nullptr;
     float4* dc = nullptr;
     int* bad = nullptr;
-    // heights on the device are read where they are (the call waits for the
-    // kernels below), host ones through a staging copy
+    // heights in this device's own memory are read where they are (the call
+    // waits for the kernels below); host ones, another device's and ones not
+    // on a float's boundary go through a staging copy
+    cudaPointerAttributes pa{};
+    const bool in_place = mem == MCRT_MEM_DEVICE && (reinterpret_cast<uintptr_t>(heights) & 3) == 0 &&
+                          cudaPointerGetAttributes(&pa, heights) == cudaSuccess &&
+                          pa.type == cudaMemoryTypeDevice && pa.device == ctx->device;
+    if (!in_place) (void)cudaGetLastError();
     const float* src = heights;
     cudaError_t e = dalloc(ctx, &dp, total * sizeof(float));
     if (e == cudaSuccess) e = dalloc(ctx, &dc, n * sizeof(float4));
     if (e == cudaSuccess) e = dalloc(ctx, &bad, sizeof(int));
-    if (e == cudaSuccess && mem == MCRT_MEM_HOST) {
+    if (e == cudaSuccess && !in_place) {
         e = dalloc(ctx, &dh, n * sizeof(float));
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dh, heights, n * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(dh, heights, n * sizeof(float),
+                                mem == MCRT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, ctx->stream);
         src = dh;
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream);

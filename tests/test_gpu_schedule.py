@@ -77,3 +77,27 @@ def test_claim_order_covers_the_image(env, size):
     a = flat.trace_camera(cam, 1, pixel_order=m.MCRT_ORDER_COST, **kw)
     b = flat.trace_camera(cam, 1, pixel_order=m.MCRT_ORDER_RASTER, **kw)
     np.testing.assert_array_equal(a.mean, b.mean)
+
+
+def test_heights_from_any_memory_are_the_same(env):
+    # in place from device memory, through a copy from the host and from an address between floats
+    import ctypes
+    import torch
+    m, ctx, sp, flat, hilly = env
+    hh = np.ascontiguousarray(scenes.heightfield(64, 0.2, seed=2)[:48, :], dtype=np.float32)
+    ny, nx = hh.shape
+    raw = torch.zeros(hh.nbytes + 2, dtype=torch.uint8, device="cuda")
+    raw[2:] = torch.from_numpy(hh.view(np.uint8).reshape(-1)).cuda()
+    xy = np.random.default_rng(0).uniform(0, 3, (500, 2)).astype(np.float32)
+    got = []
+    for how in ("host", "device", "between"):
+        sc = m.Scene.from_spec(ctx, sp)
+        if how == "between":
+            p = ctypes.c_void_p(raw.data_ptr() + 2)
+            m._check(m._load().mcrt_scene_set_ground_heightfield(sc.h, p, nx, ny, m.MCRT_MEM_DEVICE, 0.1), ctx.h)
+        else:
+            sc.set_heightfield(hh if how == "host" else torch.from_numpy(hh).cuda(), 0.1)
+        got.append(np.concatenate([np.ravel(a) for a in sc.terrain_height(xy)]))
+        sc.close()
+    np.testing.assert_array_equal(got[0], got[1])
+    np.testing.assert_array_equal(got[0], got[2])
