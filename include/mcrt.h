@@ -281,7 +281,9 @@ typedef struct {
     int32_t count_events;      /* 1: also count collisions and leaf steps       */
     int32_t rare_batch;        /* GPU lanes of a warp that must be waiting for  */
                                /* a path start, ray start or vertex before that */
-                               /* work runs (1..32; 0 = default 10).  Launch    */
+                               /* work runs (1..32; 0 = default: 20 over a      */
+                               /* heightfield and with a proposal, else 16; the */
+                               /* wavefront schedule does not use it).  Launch  */
                                /* shape only: results do not depend on it       */
     struct mcrt_proposal* proposal; /* NULL: plain HG sampling.  Else the first */
                                /* n_learned volume vertices of every path draw  */

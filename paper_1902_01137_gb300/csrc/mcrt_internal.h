@@ -225,12 +225,12 @@ struct TraceParams {
 // vertices, ended rays) once this many of its lanes wait for one (the default
 // when a caller passes 0).  Launch shape only.  A pass costs about three step
 // iterations whatever its lane count, so waiting pays until the step loop
-// runs half empty: cumulus image of 16.8 M paths 62.1, 57.3, 56.3, 57.9,
-// 64.2 ms at 8, 12, 16, 20, 24 lanes; flux of the same field 53.3, 51.7,
-// 49.9, 48.3, 52.1 ms; octree image 35.2, 32.8, 32.3, 32.9, 35.3 ms.
+// runs half empty: cumulus image of 16.8 M paths 55.6, 50.6, 48.7, 49.9,
+// 55.0 ms at 8, 12, 16, 20, 24 lanes; flux of the same field 45.5, 41.2,
+// 39.6, 40.2, 44.6 ms; octree image 31.3, 30.2, 29.8, 30.4, 32.2 ms.
 // Where a pass costs more it pays to wait longer: over a heightfield (walkers
-// wait besides) 20.0, 19.6, 19.3, 19.2 ms at 16, 18, 20, 22, in the learned
-// mode's passes 18.6, 18.5, 18.2 at 16, 18, 20.
+// wait besides) 22.6, 20.9, 19.8, 19.3, 19.3 ms, in the learned mode's
+// passes 19.6, 18.7, 18.0, 17.7, 17.9.
 constexpr int kDefaultRareBatch = 16, kDefaultRareBatchLong = 20;
 inline void set_rare_batch(TraceParams& P, int requested, bool learned = false)
 {

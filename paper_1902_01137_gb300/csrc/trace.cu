@@ -38,10 +38,11 @@
 // (no random block, sums, claims or path state in it) and its registers few
 // enough for 8 blocks of 128 threads an SM without spills; a single loop
 // with everything in it, at 72 registers and one Philox block per iteration,
-// took 95.2 ms for 16.8 M paths of the 512 x 512 x 160 cumulus image, this
-// one 56.3 ms (octree image of 11.8 M paths 46.5 -> 32.3 ms, 16.8 M flux
-// paths 81.6 -> 49.9 ms, 4 M over a relief 45.7 -> 25.4 ms).  7, 9 and 10
-// resident blocks: 56.7, 56.9 and 57.0 ms.
+// took 95.1 ms for 16.8 M paths of the 512 x 512 x 160 cumulus image, this
+// one 48.7 ms (octree image of 11.8 M paths 46.3 -> 29.8 ms, 16.8 M flux
+// paths 81.8 -> 39.5 ms, 4 M over a relief 45.6 -> 19.3 ms).  7, 9 and 10
+// resident blocks: 49.1, 48.9 and 49.1 ms (flux 40.8, 40.5, 39.3, relief
+// 19.4, 19.9, 21.6).
 // A step draws its Philox block only when its result depends on it: a
 // voxel leaf's majorant is the voxel itself, so a tentative collision there
 // is real (a sun ray's ratio 1 - k/M is 0) whatever the draw.
