@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
     };
     uint64_t t_start = 0, t_dry = 0;
     if (P.deadline_ns || COUNT) t_start = globaltimer_ns();
-    int budget = 1024;                      // step iterations until the next deadline / cancel check
+    int budget = 1024;                      // steps until the next deadline / cancel check
 
     for (;;) {
         // ==== rare pass: every lane that is not stepping ======================
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
             }
         }
         if (!__any_sync(kFull, phase != PH_IDLE)) break;
-        // ---- deadline / cancel, every 1024 step iterations --------------------
+        // ---- deadline / cancel, every 1024 steps ------------------------------
         if (budget <= 0) {
             budget = 1024;
             if (P.deadline_ns || P.cancel) {
@@ -1118,7 +1118,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
                 }
             }
             stepping = __ballot_sync(kFull, phase == PH_STEP);
-            --budget;
+            budget -= kSteps;
         } while (stepping && budget > 0 &&
                  (__popc(stepping) >= P.min_steppers || !__any_sync(kFull, phase >= PH_CLAIM)));
         mark(4);
