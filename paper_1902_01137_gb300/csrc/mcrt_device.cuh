@@ -222,6 +222,8 @@ template <bool BF16>
 __device__ __forceinline__ float brick_fetch(const DevScene& S, uint32_t brick, const int v[3], bool here, float other)
 {
 #ifdef MCRT_CHECKED
+    // (the entry's brick, which the normal build reads from, is the voxel's own)
+    MCRT_CHECK(!here || brick == (uint32_t)(brick_index(S, v[0], v[1], v[2]) >> 9), 2);
     return here ? kfetch<BF16>(S, v[0], v[1], v[2]) : other;
 #else
     const uint32_t off = ((((uint32_t)v[2] & 7u) << 3 | ((uint32_t)v[1] & 7u)) << 3) | ((uint32_t)v[0] & 7u);

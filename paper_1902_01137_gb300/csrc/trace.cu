@@ -1054,11 +1054,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
                     uint4 x = make_uint4(0u, 0u, 0u, 0u);
                     if (loads || roulette) {
                         float k = 0.0f;
-                        if (!DECOMP || loads) {
-                            const size_t idx = brick_index(Z, nv[0], nv[1], nv[2]);
-                            k = BF16 ? __uint_as_float((uint32_t)__ldg(Z.vox16 + idx) << 16) : __ldg(Z.vox + idx);
-                            k = __fadd_rn(k, Z.k_gas);
-                        }
+                        if (!DECOMP || loads) k = __fadd_rn(kfetch<BF16>(Z, nv[0], nv[1], nv[2]), Z.k_gas);
                         const uint32_t ev = geti(K_EV) & ~kTermAfter;
                         x = block(get_pid(), kind == kMain ? ev << 2 : (kind == kSunDirect ? 3u : (ev << 2) | 1u), blk);
                         ++blk;
