@@ -115,15 +115,27 @@ void pool_release(int device)
     if (g.refs > 0 && --g.refs == 0) cudaMemPoolDestroy(g.pool);
 }
 
-void pool_trim(cudaMemPool_t pool)
+cudaError_t pool_malloc(mcrt_ctx* ctx, void** p, size_t bytes)
+{
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    e = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(ctx->pool, 0);
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
+void pool_trim(mcrt_ctx* ctx)
 {
     uint64_t held = 0, used = 0;
-    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return;
-    }
-    if (held > used + kPoolKeep && cudaMemPoolTrimTo(pool, (size_t)used + kPoolKeep) != cudaSuccess) (void)cudaGetLastError();
+    cudaError_t e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &held);
+    if (e == cudaSuccess && held <= kPoolKeep) return;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used);
+    if (e == cudaSuccess && held > used + kPoolKeep) e = cudaMemPoolTrimTo(ctx->pool, (size_t)used + kPoolKeep);
+    if (e != cudaSuccess) (void)cudaGetLastError();
 }
 
 DevScene make_dev_scene(const mcrt_scene* sc, float k_gas)
@@ -333,12 +345,14 @@ int mcrt_scene_create(mcrt_ctx* ctx, const mcrt_field_desc* d, mcrt_scene** out)
     if (e != cudaSuccess) {
         dfree(ctx, sc->d_vox); dfree(ctx, sc->d_pyr); dfree(ctx, sc->d_leaf);
         delete sc;
+        pool_trim(ctx);
         return fail(ctx, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "mcrt_scene_create: %s",
                     cudaGetErrorString(e));
     }
     if (d->ext_mem == MCRT_MEM_HOST) {
         // the caller's host buffer is only borrowed for this call
         CK(ctx, cudaStreamSynchronize(ctx->stream));
+        pool_trim(ctx);
     }
     *out = sc;
     return MCRT_OK;
@@ -356,7 +370,7 @@ int mcrt_scene_destroy(mcrt_scene* sc)
     dfree(ctx, sc->d_hf);
     dfree(ctx, sc->d_hpyr);
     cudaStreamSynchronize(ctx->stream);
-    pool_trim(ctx->pool);
+    pool_trim(ctx);
     delete sc;
     return MCRT_OK;
 }
@@ -459,6 +473,7 @@ int mcrt_scene_build_octree(mcrt_scene* sc, int32_t levels)
     // replace the previous octree (its leaf map goes with it)
     if (sc->leaf_grid == MCRT_GRID_OCTREE) sc->leaf_valid = false;
     sc->gen++;
+    const PoolTrim trim(sc->d_oct ? ctx : nullptr);
     dfree(ctx, sc->d_oct);
     dfree(ctx, sc->d_oleaf);
     sc->d_oct = nullptr;
@@ -471,6 +486,7 @@ int mcrt_scene_build_octree(mcrt_scene* sc, int32_t levels)
         dfree(ctx, sc->d_oleaf);
         sc->d_oct = nullptr;
         sc->d_oleaf = nullptr;
+        pool_trim(ctx);
         return fail(ctx, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "%s: %s", who,
                     cudaGetErrorString(e));
     }
@@ -541,6 +557,7 @@ int mcrt_scene_set_ground_flat(mcrt_scene* sc, float albedo)
     if (!(albedo >= 0.0f && albedo <= 1.0f))
         return fail(sc->ctx, MCRT_ERR_ARG, "mcrt_scene_set_ground_flat: albedo must be in [0, 1]");
     sc->albedo = albedo;
+    const PoolTrim trim(sc->d_hf ? sc->ctx : nullptr);
     dfree(sc->ctx, sc->d_hf);
     dfree(sc->ctx, sc->d_hpyr);
     sc->d_hf = nullptr;
@@ -563,6 +580,7 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     if (mem != MCRT_MEM_HOST && mem != MCRT_MEM_DEVICE)
         return fail(ctx, MCRT_ERR_ARG, "%s: mem must be MCRT_MEM_HOST or MCRT_MEM_DEVICE", who);
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     // levels: 4 x 4 blocks while both sizes divide
     int lev = 1;
     while (lev < kMaxHfLevels && hnx % (1 << (2 * lev)) == 0 && hny % (1 << (2 * lev)) == 0) ++lev;
@@ -890,8 +908,7 @@ int run_wavefront(mcrt_scene* sc, TraceParams& P, const mcrt_trace_opts* o, mcrt
     unsigned long long slots = o->wavefront_slots ? (unsigned long long)o->wavefront_slots : (1ull << 21);
     if (slots > P.total) slots = P.total ? P.total : 1ull;
     WavefrontStats ws{};
-    const cudaError_t e = wavefront_camera(P, sc->storage == MCRT_STORAGE_BF16, (unsigned)slots, ctx->sm_count,
-                                           ctx->pool, ctx->stream, &ws);
+    const cudaError_t e = wavefront_camera(ctx, P, sc->storage == MCRT_STORAGE_BF16, (unsigned)slots, &ws);
     ctx->launches += ws.launches;
     if (e != cudaSuccess)
         return fail(ctx, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "%s: wavefront: %s", who,
@@ -1072,7 +1089,6 @@ int run_learned(mcrt_scene* sc, const TraceParams& P0, int sensor, const mcrt_tr
     t->kernel_ms = ms;
     int terr = 0;
     CK(ctx, tc5_take_error(&terr, ctx->stream));
-    pool_trim(ctx->pool);
     if (terr) return fail(ctx, MCRT_ERR_TIMEOUT, "%s: a tensor-core wait of the proposal network ran out", who);
     if (status == 1) return fail(ctx, MCRT_ERR_TIMEOUT, "%s: deadline of %g ms expired", who, o->deadline_ms);
     if (status == 2) return fail(ctx, MCRT_ERR_CANCELLED, "%s: cancelled", who);
@@ -1119,6 +1135,7 @@ int mcrt_trace_camera(mcrt_scene* sc, const mcrt_camera_desc* cam, uint32_t spp,
     u[2] = r[0] * f[1] - r[1] * f[0];
     const int ncells = cam->width * cam->height;
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     rc = ensure_leaf(sc, o->tau_merge, o->finest_level, o->grid);
     if (rc) return rc;
     rc = get_tally(ctx, ncells, 1, tally, who);
@@ -1215,6 +1232,7 @@ int mcrt_trace_flux(mcrt_scene* sc, uint64_t npaths, uint64_t seed, const mcrt_t
         return fail(ctx, MCRT_ERR_UNSUPPORTED, "%s: the wavefront schedule traces camera images only", who);
     if (npaths < 1) return fail(ctx, MCRT_ERR_ARG, "%s: npaths must be >= 1", who);
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     rc = ensure_leaf(sc, o->tau_merge, o->finest_level, o->grid);
     if (rc) return rc;
     rc = get_tally(ctx, 1, 3, tally, who);
@@ -1369,6 +1387,7 @@ int mcrt_trace_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, con
     bool bf16 = false;
     int rc = prepare_batch(ctx, items, n, o, who, h, total, bf16);
     if (rc) return rc;
+    const PoolTrim trim(ctx);
     rc = batch_tally(ctx, items, n, tally, who);
     if (rc) return rc;
     mcrt_tally* t = *tally;
@@ -1705,7 +1724,7 @@ int mcrt_tally_destroy(mcrt_tally* t)
     dfree(ctx, t->d_out);
     dfree(ctx, t->d_cell_n);
     cudaStreamSynchronize(ctx->stream);
-    pool_trim(ctx->pool);
+    pool_trim(ctx);
     delete t;
     return MCRT_OK;
 }
@@ -1798,6 +1817,7 @@ int mcrt_debug_dda_grid(const mcrt_scene* sc_c, const float o[3], const float d[
     for (int a = 0; a < 3; ++a)
         if (!std::isfinite(o[a])) return fail(ctx, MCRT_ERR_ARG, "mcrt_debug_dda: bad origin");
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     rc = ensure_leaf(sc, tau, finest, grid);
     if (rc) return rc;
     int* dcells = nullptr;
@@ -1836,6 +1856,7 @@ int mcrt_debug_terrain(const mcrt_scene* sc, int32_t n, const float* o, const fl
     if (n < 0 || n > (1 << 24)) return fail(ctx, MCRT_ERR_ARG, "%s: bad ray count %d", who, n);
     if (n == 0) return MCRT_OK;
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     float* buf = nullptr;
     CK(ctx, dalloc(ctx, &buf, (size_t)n * 7 * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(buf, o, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
@@ -1862,6 +1883,7 @@ int mcrt_debug_terrain_height(const mcrt_scene* sc, int32_t n, const float* xy, 
     if (n < 0 || n > (1 << 24)) return fail(ctx, MCRT_ERR_ARG, "%s: bad point count %d", who, n);
     if (n == 0) return MCRT_OK;
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     float* buf = nullptr;
     CK(ctx, dalloc(ctx, &buf, (size_t)n * 6 * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(buf, xy, (size_t)n * 2 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
@@ -1882,6 +1904,7 @@ int mcrt_debug_philox(mcrt_ctx* ctx, const uint32_t* ctr, const uint32_t* key, u
     if (!ctx || !ctr || !key || !out) return fail(ctx, MCRT_ERR_ARG, "mcrt_debug_philox: NULL argument");
     if (n == 0) return MCRT_OK;
     CK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     uint32_t *dc = nullptr, *dk = nullptr, *dout = nullptr;
     CK(ctx, dalloc(ctx, &dc, n * 16));
     CK(ctx, dalloc(ctx, &dk, n * 8));

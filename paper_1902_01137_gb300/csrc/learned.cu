@@ -126,7 +126,7 @@ int mcrt_proposal_destroy(mcrt_proposal* P)
                     (void*)P->d_bias})
         if (p) cudaFreeAsync(p, ctx->stream);
     cudaStreamSynchronize(ctx->stream);
-    pool_trim(ctx->pool);
+    pool_trim(ctx);
     delete P;
     return MCRT_OK;
 }
@@ -213,6 +213,7 @@ int mcrt_proposal_eval(mcrt_proposal* P, const float* host_feat, size_t n, float
     if (n == 0) return MCRT_OK;
     if (n > (size_t)(1 << 28)) return lfail(ctx, MCRT_ERR_ARG, "mcrt_proposal_eval: too many rows");
     LCK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     float* d_f32 = nullptr;
     void* d_feat = nullptr;
     float *d_mix = nullptr, *d_raw = nullptr;
@@ -251,6 +252,7 @@ int mcrt_proposal_train_step(mcrt_proposal* P, const float* host_feat, const flo
     if (n == 0 || n > (size_t)(1 << 26)) return lfail(ctx, MCRT_ERR_ARG, "mcrt_proposal_train_step: bad record count");
     if (!(lr >= 0.0f)) return lfail(ctx, MCRT_ERR_ARG, "mcrt_proposal_train_step: lr must be >= 0");
     LCK(ctx, cudaSetDevice(ctx->device));
+    const PoolTrim trim(ctx);
     float *d_f32 = nullptr, *d_dirs = nullptr, *d_t = nullptr;
     void* d_feat = nullptr;
     LCK(ctx, pool_alloc(ctx, &d_f32, n * 9 * sizeof(float)));

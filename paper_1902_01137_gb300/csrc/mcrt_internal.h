@@ -123,20 +123,32 @@ namespace mcrt {
 // Device memory.  The contexts of a device share one stream-ordered pool of
 // the library's own, made with the first context and destroyed with the
 // last.  Freed memory stays in it, up to kPoolKeep bytes beyond what is in
-// use (pool_trim, called where objects and workspaces are given back): the
-// device's default pool hands every freed byte back to the driver at the next
-// synchronisation, and mapping it again cost a learned image of 4.2 M paths
-// 3.5 ms a call and a 671 MB field's scene 2 ms.  The pool calls are safe from
-// several threads and streams.
+// use: the device's default pool hands every freed byte back to the driver at
+// the next synchronisation, and mapping it again cost a learned image of 4.2 M
+// paths 3.5 ms a call and a 671 MB field's scene 2 ms.  Every call that frees
+// memory ends with pool_trim (PoolTrim: whichever way it ends), which waits
+// for the context's stream, since frees count only once done, but only where
+// the pool holds more than kPoolKeep at all.  An allocation that finds no
+// memory gives back what the pool keeps and tries again.  The pool calls are
+// safe from several threads and streams.
 constexpr size_t kPoolKeep = (size_t)4 << 30;
 cudaError_t pool_acquire(int device, cudaMemPool_t* pool);
 void pool_release(int device);
-void pool_trim(cudaMemPool_t pool);
+cudaError_t pool_malloc(mcrt_ctx* ctx, void** p, size_t bytes);
+void pool_trim(mcrt_ctx* ctx);
+
+struct PoolTrim {
+    mcrt_ctx* ctx;             // null: nothing to do
+    explicit PoolTrim(mcrt_ctx* c) : ctx(c) {}
+    ~PoolTrim() { if (ctx) pool_trim(ctx); }
+    PoolTrim(const PoolTrim&) = delete;
+    PoolTrim& operator=(const PoolTrim&) = delete;
+};
 
 template <class T>
 cudaError_t pool_alloc(mcrt_ctx* ctx, T** p, size_t bytes)
 {
-    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes == 0 ? 16 : bytes, ctx->pool, ctx->stream);
+    return pool_malloc(ctx, reinterpret_cast<void**>(p), bytes == 0 ? 16 : bytes);
 }
 
 constexpr int kNumCounters = 32;
@@ -330,8 +342,7 @@ struct WavefrontStats {
     unsigned overflow;             // 1: a queue was full; 2: too many rounds
     unsigned long long launches;
 };
-cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, int sm_count, cudaMemPool_t pool,
-                             cudaStream_t st, WavefrontStats* stats);
+cudaError_t wavefront_camera(mcrt_ctx* ctx, const TraceParams& P, bool bf16, unsigned slots, WavefrontStats* stats);
 int wavefront_blocks_per_sm(bool bf16);
 
 // Option checks shared by the trace entry points (status and message as

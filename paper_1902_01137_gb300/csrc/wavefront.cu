@@ -567,9 +567,9 @@ int wavefront_blocks_per_sm(bool bf16)
     return std::max(1, std::min(a, b));
 }
 
-cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, int sm_count, cudaMemPool_t pool,
-                             cudaStream_t st, WavefrontStats* stats)
+cudaError_t wavefront_camera(mcrt_ctx* ctx, const TraceParams& P, bool bf16, unsigned slots, WavefrontStats* stats)
 {
+    const cudaStream_t st = ctx->stream;
     *stats = WavefrontStats{};
     const unsigned cap = slots;
     WfParams W{};
@@ -577,13 +577,13 @@ cudaError_t wavefront_camera(const TraceParams& P, bool bf16, unsigned slots, in
     W.cap = cap;
     char* buf = nullptr;
     const size_t qb = queue_bytes(cap);
-    cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&buf), 3 * qb + 256, pool, st);
+    cudaError_t e = pool_alloc(ctx, &buf, 3 * qb + 256);
     if (e != cudaSuccess) return e;
     carve(W.F[0], buf, cap);
     carve(W.F[1], buf + qb, cap);
     carve(W.V, buf + 2 * qb, cap);
     W.st = reinterpret_cast<WfState*>(buf + 3 * qb);
-    const int grid = sm_count * wavefront_blocks_per_sm(bf16);
+    const int grid = ctx->sm_count * wavefront_blocks_per_sm(bf16);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
