@@ -599,15 +599,6 @@ MCRT_API int mcrt_debug_terrain_height(const mcrt_scene* scene, int32_t n, const
 MCRT_API int mcrt_debug_bounds_violations(mcrt_ctx* ctx, int32_t* checked_build, uint64_t* count,
                                           int32_t* first_code);
 
-/* Device memory held by the allocations of the library's stream-ordered
- * memory pool on the context's device (the pool every allocation of this
- * library draws from, except a batch plan's item table; shared by the
- * device's contexts, destroyed with the last, and keeping at most 4 GiB that
- * nothing uses): *used_current now and
- * *used_high the most since the last reset; reset_high != 0 then resets the
- * high mark to the current use.  Lets a caller check that a call allocated
- * nothing (the paper has no counterpart).  Synchronises the context
- * stream. */
 /* The online-training records of one learned trace, for checks against an
  * independent implementation: the trace runs as mcrt_trace_camera
  * (camera != NULL, n = samples per pixel) or mcrt_trace_flux (n paths) with
@@ -627,6 +618,15 @@ MCRT_API int mcrt_debug_learned_records(mcrt_scene* scene, const mcrt_camera_des
                                         const mcrt_trace_opts* opts, int32_t cap, float* feat, float* dir,
                                         float* val, uint64_t* path, int32_t* count);
 
+/* Device memory held by the library's allocations, all from one
+ * stream-ordered memory pool except a batch plan's item table: *used_current
+ * now and *used_high the most since the last reset; reset_high != 0 then
+ * resets the high mark to the current use.  The pool is the one the program
+ * has made the device's current one (cudaDeviceSetMemPool), under that pool's
+ * bounds, and where it has set none the library's own on the device: shared
+ * by the device's contexts, destroyed with the last, and keeping at most
+ * 4 GiB that nothing uses.  Lets a caller check that a call allocated nothing
+ * (the paper has no counterpart).  Synchronises the context stream. */
 MCRT_API int mcrt_debug_pool_usage(mcrt_ctx* ctx, int32_t reset_high, uint64_t* used_current, uint64_t* used_high);
 
 /* Philox4x32-10 evaluated on the device for n (counter[4], key[2]) pairs

@@ -450,9 +450,10 @@ def mcrt_debug_learned_records(ctx, scene, cam, n: int, seed: int, opts, cap: in
 
 
 def mcrt_debug_pool_usage(ctx, reset_high: bool = False):
-    """(bytes in use, most bytes in use since the last reset) of the library's
-    stream-ordered memory pool on the device; reset_high then resets the high
-    mark."""
+    """(bytes in use, most bytes in use since the last reset) of the
+    stream-ordered memory pool the library allocates from: the program's own
+    where it has set one for the device, else the library's; reset_high then
+    resets the high mark."""
     cur, high = C.c_uint64(), C.c_uint64()
     _check(_load().mcrt_debug_pool_usage(ctx, 1 if reset_high else 0, C.byref(cur), C.byref(high)), ctx)
     return int(cur.value), int(high.value)

@@ -115,14 +115,23 @@ void pool_release(int device)
     if (g.refs > 0 && --g.refs == 0) cudaMemPoolDestroy(g.pool);
 }
 
+cudaMemPool_t pool_current(const mcrt_ctx* ctx)
+{
+    cudaMemPool_t cur = nullptr;
+    if (cudaDeviceGetMemPool(&cur, ctx->device) == cudaSuccess) return cur == ctx->default_pool ? ctx->pool : cur;
+    (void)cudaGetLastError();
+    return ctx->pool;
+}
+
 cudaError_t pool_malloc(mcrt_ctx* ctx, void** p, size_t bytes)
 {
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    const cudaMemPool_t pool = pool_current(ctx);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, ctx->stream);
     if (e != cudaErrorMemoryAllocation) return e;
     (void)cudaGetLastError();
     e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) e = cudaMemPoolTrimTo(ctx->pool, 0);
-    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, ctx->stream);
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;
 }
@@ -234,7 +243,8 @@ int mcrt_create(mcrt_ctx** out, int device, void* cuda_stream)
         return fail(nullptr, MCRT_ERR_CUDA, "mcrt_create: %s", cudaGetErrorString(e));
     }
     c->l2_bytes = (size_t)l2;
-    e = pool_acquire(device, &c->pool);
+    e = cudaDeviceGetDefaultMemPool(&c->default_pool, device);
+    if (e == cudaSuccess) e = pool_acquire(device, &c->pool);
     if (e != cudaSuccess) {
         delete c;
         return fail(nullptr, e == cudaErrorMemoryAllocation ? MCRT_ERR_OOM : MCRT_ERR_CUDA, "mcrt_create: memory pool: %s",
@@ -1778,7 +1788,7 @@ int mcrt_debug_pool_usage(mcrt_ctx* ctx, int32_t reset_high, uint64_t* used_curr
     if (!ctx || !used_current || !used_high) return fail(ctx, MCRT_ERR_ARG, "mcrt_debug_pool_usage: NULL argument");
     CK(ctx, cudaSetDevice(ctx->device));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
-    const cudaMemPool_t pool = ctx->pool;
+    const cudaMemPool_t pool = pool_current(ctx);
     unsigned long long cur = 0, high = 0;
     CK(ctx, cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &cur));
     CK(ctx, cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &high));

@@ -38,6 +38,7 @@ struct mcrt_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaMemPool_t pool = nullptr;     // the device's library pool (pool_acquire)
+    cudaMemPool_t default_pool = nullptr;   // the driver's, current unless the program sets another
     int sm_count = 0;
     size_t l2_bytes = 0;
     uint64_t launches = 0;
@@ -120,7 +121,9 @@ struct mcrt_proposal {
 
 namespace mcrt {
 
-// Device memory.  The contexts of a device share one stream-ordered pool of
+// Device memory.  Where the program has made a pool of its own the device's
+// current one (cudaDeviceSetMemPool), allocations draw from that, under its
+// bounds.  Otherwise the contexts of a device share one stream-ordered pool of
 // the library's own, made with the first context and destroyed with the
 // last.  Freed memory stays in it, up to kPoolKeep bytes beyond what is in
 // use: the device's default pool hands every freed byte back to the driver at
@@ -134,6 +137,7 @@ namespace mcrt {
 constexpr size_t kPoolKeep = (size_t)4 << 30;
 cudaError_t pool_acquire(int device, cudaMemPool_t* pool);
 void pool_release(int device);
+cudaMemPool_t pool_current(const mcrt_ctx* ctx);
 cudaError_t pool_malloc(mcrt_ctx* ctx, void** p, size_t bytes);
 void pool_trim(mcrt_ctx* ctx);
 

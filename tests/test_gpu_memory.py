@@ -115,3 +115,67 @@ def test_replaced_heightfields_are_given_back(env):
             m.mcrt_scene_set_ground_flat(ctx.h, sc.h, 0.1)
         sc.close()
     assert held.unused <= KEEP + SLACK
+
+
+class ProgramPool:
+    """A memory pool of the program's own, current for device 0 meanwhile."""
+
+    USED_NOW = 7                                    # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+
+    def __init__(self, max_bytes=0):
+        self.cu = C.CDLL("libcuda.so.1")
+        self.max_bytes = max_bytes
+
+    def _ok(self, rc):
+        assert rc == 0, rc
+
+    def __enter__(self):
+        class Props(C.Structure):                   # CUmemPoolProps
+            _fields_ = [("alloc_type", C.c_int), ("handle_types", C.c_int), ("loc_type", C.c_int), ("loc_id", C.c_int),
+                        ("security", C.c_void_p), ("max_size", C.c_size_t), ("usage", C.c_ushort),
+                        ("reserved", C.c_ubyte * 54)]
+        p = Props(alloc_type=1, loc_type=1, loc_id=0, max_size=self.max_bytes)      # pinned, on the device
+        self.pool, self.default = C.c_void_p(), C.c_void_p()
+        self._ok(self.cu.cuDeviceGetDefaultMemPool(C.byref(self.default), 0))
+        self._ok(self.cu.cuMemPoolCreate(C.byref(self.pool), C.byref(p)))
+        self._ok(self.cu.cuDeviceSetMemPool(0, self.pool))
+        return self
+
+    def used(self):
+        v = C.c_uint64()
+        self._ok(self.cu.cuMemPoolGetAttribute(self.pool, self.USED_NOW, C.byref(v)))
+        return v.value
+
+    def __exit__(self, *a):
+        self._ok(self.cu.cuDeviceSetMemPool(0, self.default))
+        self._ok(self.cu.cuMemPoolDestroy(self.pool))
+
+
+@pytest.mark.parametrize("first", ["context", "pool"])
+def test_the_programs_own_pool_is_used(env, first):
+    torch, m = env
+    sp = scenes.blobs_small(0)
+    cam = scenes.nadir_camera(sp, 16, 16)
+    before = m.Context(0) if first == "context" else None
+    with ProgramPool() as pool:
+        ctx = before or m.Context(0)
+        sc = m.Scene.from_spec(ctx, sp)
+        assert pool.used() >= sp.k.nbytes
+        assert m.mcrt_debug_pool_usage(ctx.h)[0] == pool.used()
+        want = sc.trace_camera(cam, 4, seed=1).mean
+        sc.close()
+        assert pool.used() == 0
+    sc = m.Scene.from_spec(ctx, sp)
+    np.testing.assert_allclose(sc.trace_camera(cam, 4, seed=1).mean, want, rtol=1e-12, atol=0)
+    sc.close()
+    ctx.close()
+
+
+def test_the_programs_bound_holds(env):
+    torch, m = env
+    with ProgramPool(max_bytes=64 << 20), m.Context(0) as ctx:
+        k = torch.ones((128, 512, 512), device="cuda")
+        with pytest.raises(m.McrtError) as e:
+            m.Scene(ctx, k, 0.1, 0.1, 0.1)
+        assert e.value.status == m.MCRT_ERR_OOM
+        m.Scene(ctx, k[:8, :64, :64], 0.1, 0.1, 0.1).close()
