@@ -123,6 +123,12 @@ MCRT_API const char* mcrt_last_error(const mcrt_ctx* ctx);
 /* Number of kernels this context has launched so far (all calls). */
 MCRT_API int mcrt_launch_count(const mcrt_ctx* ctx, uint64_t* count);
 
+/* Give back to the driver all the device memory that the library keeps and
+ * nothing uses (at most 4 GiB on the device; the next calls map it again).
+ * Waits for the context's stream.  A pool of the program's own
+ * (mcrt_debug_pool_usage) is left to the program. */
+MCRT_API int mcrt_trim_memory(mcrt_ctx* ctx);
+
 /* --------------------------------------------------------------------- */
 /* Scene: the extinction field, its majorant pyramid, ground and sun.     */
 /* --------------------------------------------------------------------- */

@@ -120,6 +120,7 @@ def _load():
         "mcrt_destroy": [vp],
         "mcrt_last_error": [vp],
         "mcrt_launch_count": [vp, P(u64)],
+        "mcrt_trim_memory": [vp],
         "mcrt_scene_create": [vp, P(FieldDesc), P(vp)],
         "mcrt_scene_destroy": [vp],
         "mcrt_scene_build_majorants": [vp, i32],
@@ -236,6 +237,12 @@ def mcrt_launch_count(ctx) -> int:
     v = C.c_uint64()
     _check(_load().mcrt_launch_count(ctx, C.byref(v)), ctx)
     return v.value
+
+
+def mcrt_trim_memory(ctx):
+    """Give the device memory that the library keeps and nothing uses (at
+    most 4 GiB) back to the driver."""
+    _check(_load().mcrt_trim_memory(ctx), ctx)
 
 
 def mcrt_scene_create(ctx, desc: FieldDesc):
@@ -490,6 +497,9 @@ class Context:
     @property
     def launches(self) -> int:
         return mcrt_launch_count(self.h)
+
+    def trim_memory(self):
+        mcrt_trim_memory(self.h)
 
 
 @dataclass

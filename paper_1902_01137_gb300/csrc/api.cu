@@ -275,6 +275,15 @@ int mcrt_launch_count(const mcrt_ctx* ctx, uint64_t* count)
     return MCRT_OK;
 }
 
+int mcrt_trim_memory(mcrt_ctx* ctx)
+{
+    if (!ctx) return fail(nullptr, MCRT_ERR_ARG, "mcrt_trim_memory: NULL context");
+    CK(ctx, cudaSetDevice(ctx->device));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    CK(ctx, cudaMemPoolTrimTo(ctx->pool, 0));
+    return MCRT_OK;
+}
+
 // ---------------------------------------------------------------------------
 // Scene
 // ---------------------------------------------------------------------------

@@ -179,3 +179,19 @@ def test_the_programs_bound_holds(env):
             m.Scene(ctx, k, 0.1, 0.1, 0.1)
         assert e.value.status == m.MCRT_ERR_OOM
         m.Scene(ctx, k[:8, :64, :64], 0.1, 0.1, 0.1).close()
+
+
+def test_kept_memory_is_given_back_on_request(env):
+    torch, m = env
+    with m.Context(0) as ctx:
+        sc = m.Scene.from_spec(ctx, scenes.blobs_small(0))
+        with Held(env, ctx) as held:
+            m.Scene(ctx, torch.zeros((512, 1024, 1024), device="cuda"), 0.1, 0.1, 0.1, levels=1).close()
+            torch.cuda.empty_cache()
+            kept = torch.cuda.mem_get_info()[0]
+            ctx.trim_memory()
+            given = torch.cuda.mem_get_info()[0] - kept
+        assert given >= 2 << 30
+        assert held.unused <= SLACK
+        assert sc.trace_flux(1000, seed=1).mean[0] > 0.0      # (what is in use stays)
+        sc.close()
