@@ -429,11 +429,14 @@ MCRT_API int mcrt_trace_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32
 
 /* Launch-shape autotuner for a batch: times mcrt_trace_batch on a fraction
  * of every item's paths for each candidate (paths per claim 1, 2, 4, 8;
- * rare-phase wait 4, 8, 12 lanes; 64 or 128 threads per block; the better
- * of two runs each) and writes the fastest into *opts_inout (*best_ms: its
- * time).  Too small a fraction lets the last, straggling paths dominate;
- * a quarter of the paths or more tunes for the full batch.  Results of a trace do
- * not depend on these choices, only its speed. */
+ * rare-phase wait 12, 16, 20, 24 lanes; 64 or 128 threads per block; then
+ * the shape in *opts_inout, where it sets any of these or a grid size; the
+ * better of two runs each) and writes the fastest into *opts_inout
+ * (*best_ms: its time).  A batch of at most 8 paths a warp never waits: one
+ * wait, 12 lanes, is tried; a larger one with a sample that small keeps the
+ * default wait.  Too small a fraction lets the last, straggling paths
+ * dominate; a quarter of the paths or more tunes for the full batch.
+ * Results of a trace do not depend on these choices, only its speed. */
 MCRT_API int mcrt_autotune_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, double path_fraction,
                                  mcrt_trace_opts* opts_inout, float* best_ms);
 

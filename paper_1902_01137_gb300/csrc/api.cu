@@ -1453,27 +1453,54 @@ int mcrt_autotune_batch(mcrt_ctx* ctx, const mcrt_batch_item* items, int32_t n, 
         it.npaths = (uint64_t)std::ceil((double)it.npaths * path_fraction);
         if (it.npaths < 1) it.npaths = 1;
     }
-    // candidate launch shapes: paths per claim x lanes a rare phase waits for x block size
+    // Candidate launch shapes: block size x paths per claim x lanes a rare pass
+    // waits for, around the defaults (128, 4, 16), and the caller's own shape.
+    // The wait is measured only where there is one: of at most 8 paths a warp,
+    // with their sun rays on helpers, 16 lanes step, and a pass is put off only
+    // above 32 - wait of them, so up to 16 every wait gives the same launch, and
+    // a longer one only holds up a launch that its longest paths bound.  A sample
+    // that thin of a batch that is not says nothing about the wait.
+    const mcrt_trace_opts mine = *opts_inout;
     const int chunks[] = {1, 2, 4, 8};
-    const int rares[] = {4, 8, 12};
     const int blocks[] = {64, 128};
-    mcrt_tally* t = nullptr;
-    float best = 3.0e38f;
-    mcrt_trace_opts bo = *opts_inout;
+    CK(ctx, cudaSetDevice(ctx->device));
+    const unsigned long long warps =
+        (unsigned long long)ctx->sm_count * 4 *
+        trace_batch_blocks_per_sm(false, mine.count_events != 0, mine.batch_dalpha != 0, 128);
+    auto thin = [&](const mcrt_batch_item* its) {
+        unsigned long long paths = 0;
+        for (int i = 0; i < n; ++i) paths += its[i].npaths;
+        return paths <= 8 * warps;
+    };
+    std::vector<int> rares = {12, 16, 20, 24};
+    if (thin(items)) rares = {12};
+    else if (thin(sub.data())) rares = {kDefaultRareBatch};
+    std::vector<mcrt_trace_opts> shapes;
     for (int b : blocks)
         for (int c : chunks)
             for (int r : rares) {
-                mcrt_trace_opts o = *opts_inout;
+                mcrt_trace_opts o = mine;
                 o.chunk = c;
                 o.rare_batch = r;
                 o.block_size = b;
                 o.grid_size = 0;
-                for (int rep = 0; rep < 2; ++rep) {          // the better of two runs
-                    int rc = mcrt_trace_batch(ctx, sub.data(), n, &o, &t);
-                    if (rc) { if (t) mcrt_tally_destroy(t); return rc; }
-                    if (t->kernel_ms < best) { best = t->kernel_ms; bo = o; }
-                }
+                shapes.push_back(o);
             }
+    const size_t own = shapes.size();
+    if (mine.chunk || mine.rare_batch || mine.block_size || mine.grid_size) shapes.push_back(mine);
+    mcrt_tally* t = nullptr;
+    float best = 3.0e38f;
+    mcrt_trace_opts bo = mine;
+    for (size_t q = 0; q < shapes.size(); ++q)
+        for (int rep = 0; rep < 2; ++rep) {              // the better of two runs
+            int rc = mcrt_trace_batch(ctx, sub.data(), n, &shapes[q], &t);
+            if (q == own && (rc == MCRT_ERR_ARG || rc == MCRT_ERR_UNSUPPORTED)) {
+                ctx->err.clear();                        // no shape a trace takes: the others stand
+                break;
+            }
+            if (rc) { if (t) mcrt_tally_destroy(t); return rc; }
+            if (t->kernel_ms < best) { best = t->kernel_ms; bo = shapes[q]; }
+        }
     if (t) mcrt_tally_destroy(t);
     *opts_inout = bo;
     if (best_ms) *best_ms = best;
