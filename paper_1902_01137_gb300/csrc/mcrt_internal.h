@@ -84,7 +84,8 @@ struct mcrt_scene {
     float sun_zenith = 0, sun_azimuth = 0;
     float sun[3] = {0, 0, 1};
     // heightfield ground (null: flat)
-    float4* d_hf = nullptr;
+    float* d_hf = nullptr;            // a record of four corners per cell ...
+    bool hf_rec = false;              // ... or, past kHfRecordCells, the plain heights
     float* d_hpyr = nullptr;
     int hn[2] = {0, 0};
     float hmax = 0;
@@ -154,6 +155,16 @@ cudaError_t pool_alloc(mcrt_ctx* ctx, T** p, size_t bytes)
 {
     return pool_malloc(ctx, reinterpret_cast<void**>(p), bytes == 0 ? 16 : bytes);
 }
+
+// Heightfields of at most this many cells (16,384^2: 4.3 GB of records) are kept
+// as one 16-byte record of corners per cell, larger ones as the plain 4-byte
+// heights, so that a relief that fits beside its field by those still does.
+// 4 M flux paths: 19.2 ms with records, 20.3 with heights over 4096^2 cells,
+// 33.6 and 35.0 over 20,000^2.
+#ifndef MCRT_HF_RECORD_CELLS
+#define MCRT_HF_RECORD_CELLS (1ll << 28)
+#endif
+constexpr long long kHfRecordCells = MCRT_HF_RECORD_CELLS;
 
 constexpr int kNumCounters = 32;
 constexpr int kMlpParams = 11560;
@@ -280,13 +291,13 @@ cudaError_t launch_reduce_level(const float* pmax, const float* pmin, const int*
 cudaError_t launch_leafmap(const mcrt_scene* sc, float tau, int finest, int grid, cudaStream_t st);
 cudaError_t launch_octree(const mcrt_scene* sc, cudaStream_t st);
 cudaError_t launch_hf_pyramid(const float* h, int nx, int ny, float4* cells, float* pyr, const int* off, int levels,
-                              cudaStream_t st);
+                              cudaStream_t st);   // cells null: no records
 cudaError_t launch_hf_check(const float* h, long long n, float top, int* bad, cudaStream_t st);
 cudaError_t launch_debug_terrain(const DevScene& S, const float* o, const float* d, int n, float* t, cudaStream_t st);
 cudaError_t launch_debug_terrain_height(const DevScene& S, const float* xy, int n, float* zn, cudaStream_t st);
 cudaError_t launch_trace(const TraceParams& P, int sensor, bool bf16, bool count, int grid, int block,
                          cudaStream_t st);
-int trace_blocks_per_sm(int sensor, bool bf16, bool count, bool terrain, bool extra, int block);
+int trace_blocks_per_sm(int sensor, bool bf16, bool count, const DevScene& S, bool extra, int block);
 cudaError_t launch_trace_learned(const TraceParams& P, int sensor, bool bf16, int grid, int block, cudaStream_t st);
 int trace_learned_blocks_per_sm(int sensor, bool bf16, int block);
 cudaError_t launch_targets(const float* rec_val, const float* final_score, unsigned n, float* tgt, cudaStream_t st);

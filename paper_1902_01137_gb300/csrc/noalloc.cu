@@ -186,7 +186,7 @@ extern "C" int mcrt_trace_camera_noalloc(mcrt_scene* sc, const mcrt_camera_desc*
     const bool bf16 = sc->storage == MCRT_STORAGE_BF16;
     const bool count = o->count_events != 0;
     const int block = o->block_size ? o->block_size : 128;
-    const int grid = o->grid_size ? o->grid_size : ctx->sm_count * trace_blocks_per_sm(kCamera, bf16, count, P.S.hf != nullptr, P.sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh, block);
+    const int grid = o->grid_size ? o->grid_size : ctx->sm_count * trace_blocks_per_sm(kCamera, bf16, count, P.S, P.sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh, block);
     if (!o->chunk) P.chunk = auto_chunk(P.total, ctx->sm_count, o->grid_size, block, spp);
     set_claim_lanes(P, grid, block);
     ctx->launches++;

@@ -145,6 +145,9 @@ constexpr uint32_t kMaxHelpers = 5;
 // cycles per vertex with a helper, 8,000 without; 64 x 64 x 16 paths of the
 // blob field 2.5 -> 2.05 ms, a 500 x 301 x 16 image 10.5 -> 9.3 ms.
 
+// The ground: flat, or a heightfield in either of its forms (DevScene::hf).
+enum Ground { kFlat = 0, kRecords, kHeights };
+
 // A batch's kernel holds its lane's scene pointer and derivative sums besides:
 // 12 fields 89.6 ms with spills at 8 blocks of 128, 88.0 without at 7.
 constexpr int kBatchBlocks = 7;
@@ -152,9 +155,8 @@ constexpr int kBatchBlocks = 7;
 // EXTRA: the variants that also handle decomposition tracking of sun rays
 // and Rayleigh clear air (chosen at run time); the others carry neither, so
 // the paper's estimator keeps its registers.  In batches, EXTRA instead
-// adds the dT/dalpha estimate.
-template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, bool BATCH = false, bool TERRAIN = false,
-          bool EXTRA = false>
+// adds the dT/dalpha estimate.  TERRAIN: the ground (Ground).
+template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, bool BATCH = false, int TERRAIN = kFlat, bool EXTRA = false>
 __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLOCKS) trace_kernel(const __grid_constant__ TraceParams P)
 {
     // Steps between looks at who waits.  Two spare half of the votes and the
@@ -708,7 +710,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
                     // irradiance of the tilted element per horizontal area is
                     // max(n.s, 0) / (n_z mu0) T_sun, kept in tdir until T_sun
                     float n[3];
-                    vx[2] = hf_height(S, vx[0], vx[1], n);
+                    vx[2] = hf_height<TERRAIN == kRecords>(S, vx[0], vx[1], n);
 #pragma unroll
                     for (int a = 0; a < 3; ++a) vx[a] += kTerrainOffset * n[a];
 #pragma unroll
@@ -767,7 +769,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
                 // tilted ground: leave the surface along its normal, estimate
                 // with n.s, scatter cosine-weighted about n
                 float n[3];
-                hf_height(S, vx[0], vx[1], n);
+                hf_height<TERRAIN == kRecords>(S, vx[0], vx[1], n);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) vx[a] += kTerrainOffset * n[a];
 #pragma unroll
@@ -984,7 +986,7 @@ __global__ void __launch_bounds__(128, BATCH ? kBatchBlocks : MCRT_TRACE_MIN_BLO
             const int steppers = __popc(__ballot_sync(kFull, phase == PH_STEP));
             if (__popc(walkers) >= kWalkBatch || (walkers && steppers < P.min_steppers)) {
                 if (phase == PH_WALK) {
-                    const float th = terrain_hit(Z, R.o, R.d);
+                    const float th = terrain_hit<TERRAIN == kRecords>(Z, R.o, R.d);
                     phase = PH_STEP;
                     if (kind == kMain) {
                         tg = th;
@@ -1368,7 +1370,7 @@ __global__ void debug_terrain_kernel(DevScene S, const float* __restrict__ o, co
     if (i >= n) return;
     const float oo[3] = {o[3 * i], o[3 * i + 1], o[3 * i + 2]};
     const float dd[3] = {d[3 * i], d[3 * i + 1], d[3 * i + 2]};
-    t[i] = terrain_hit(S, oo, dd);
+    t[i] = S.hrec ? terrain_hit<true>(S, oo, dd) : terrain_hit<false>(S, oo, dd);
 }
 
 // One thread per point: surface height and normal (z, nx, ny, nz).
@@ -1377,7 +1379,7 @@ __global__ void debug_terrain_height_kernel(DevScene S, const float* __restrict_
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float nn[3];
-    zn[4 * i] = hf_height(S, xy[2 * i], xy[2 * i + 1], nn);
+    zn[4 * i] = S.hrec ? hf_height<true>(S, xy[2 * i], xy[2 * i + 1], nn) : hf_height<false>(S, xy[2 * i], xy[2 * i + 1], nn);
     zn[4 * i + 1] = nn[0]; zn[4 * i + 2] = nn[1]; zn[4 * i + 3] = nn[2];
 }
 
@@ -1391,13 +1393,13 @@ __global__ void debug_philox_kernel(const uint32_t* __restrict__ ctr, const uint
     out[4 * i] = r.x; out[4 * i + 1] = r.y; out[4 * i + 2] = r.z; out[4 * i + 3] = r.w;
 }
 
-template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, bool TERRAIN = false, bool EXTRA = false>
+template <int SENSOR, bool BF16, bool COUNT, bool LEARNED, int TERRAIN = kFlat, bool EXTRA = false>
 const void* kernel_ptr()
 {
     return reinterpret_cast<const void*>(&trace_kernel<SENSOR, BF16, COUNT, LEARNED, false, TERRAIN, EXTRA>);
 }
 
-template <bool TERRAIN, bool DECOMP>
+template <int TERRAIN, bool DECOMP>
 const void* pick_t(int sensor, bool bf16, bool count)
 {
     if (sensor == kCamera) {
@@ -1415,20 +1417,26 @@ const void* pick_t(int sensor, bool bf16, bool count)
 // Kernel of a plain trace: sensor, storage, counting, heightfield ground and
 // whether decomposition tracking or Rayleigh clear air is in use (those have
 // variants of their own, so the others keep their registers).
-const void* pick(int sensor, bool bf16, bool count, bool terrain, bool extra)
+template <bool EXTRA>
+const void* pick_g(int sensor, bool bf16, bool count, const DevScene& S)
 {
-    if (extra) return terrain ? pick_t<true, true>(sensor, bf16, count) : pick_t<false, true>(sensor, bf16, count);
-    return terrain ? pick_t<true, false>(sensor, bf16, count) : pick_t<false, false>(sensor, bf16, count);
+    if (!S.hf) return pick_t<kFlat, EXTRA>(sensor, bf16, count);
+    return S.hrec ? pick_t<kRecords, EXTRA>(sensor, bf16, count) : pick_t<kHeights, EXTRA>(sensor, bf16, count);
+}
+
+const void* pick(int sensor, bool bf16, bool count, const DevScene& S, bool extra)
+{
+    return extra ? pick_g<true>(sensor, bf16, count, S) : pick_g<false>(sensor, bf16, count, S);
 }
 
 template <bool DALPHA>
 const void* pick_batch_t(bool bf16, bool count)
 {
     if (count)
-        return bf16 ? reinterpret_cast<const void*>(&trace_kernel<kFlux, true, true, false, true, false, DALPHA>)
-                    : reinterpret_cast<const void*>(&trace_kernel<kFlux, false, true, false, true, false, DALPHA>);
-    return bf16 ? reinterpret_cast<const void*>(&trace_kernel<kFlux, true, false, false, true, false, DALPHA>)
-                : reinterpret_cast<const void*>(&trace_kernel<kFlux, false, false, false, true, false, DALPHA>);
+        return bf16 ? reinterpret_cast<const void*>(&trace_kernel<kFlux, true, true, false, true, kFlat, DALPHA>)
+                    : reinterpret_cast<const void*>(&trace_kernel<kFlux, false, true, false, true, kFlat, DALPHA>);
+    return bf16 ? reinterpret_cast<const void*>(&trace_kernel<kFlux, true, false, false, true, kFlat, DALPHA>)
+                : reinterpret_cast<const void*>(&trace_kernel<kFlux, false, false, false, true, kFlat, DALPHA>);
 }
 
 const void* pick_batch(bool bf16, bool count, bool dalpha)
@@ -1463,7 +1471,7 @@ cudaError_t launch_trace(const TraceParams& P, int sensor, bool bf16, bool count
 {
     void* args[] = {const_cast<TraceParams*>(&P)};
     const bool extra = P.sun_mode == MCRT_SUN_DECOMP || P.S.rayleigh;
-    return cudaLaunchKernel(pick(sensor, bf16, count, P.S.hf != nullptr, extra), dim3(grid), dim3(block), args, 0, st);
+    return cudaLaunchKernel(pick(sensor, bf16, count, P.S, extra), dim3(grid), dim3(block), args, 0, st);
 }
 
 cudaError_t launch_trace_learned(const TraceParams& P, int sensor, bool bf16, int grid, int block, cudaStream_t st)
@@ -1501,10 +1509,10 @@ cudaError_t launch_targets(const float* rec_val, const float* final_score, unsig
     return cudaGetLastError();
 }
 
-int trace_blocks_per_sm(int sensor, bool bf16, bool count, bool terrain, bool extra, int block)
+int trace_blocks_per_sm(int sensor, bool bf16, bool count, const DevScene& S, bool extra, int block)
 {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pick(sensor, bf16, count, terrain, extra), block, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pick(sensor, bf16, count, S, extra), block, 0) !=
         cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
