@@ -12,6 +12,9 @@
 #include <vector>
 #include <utility>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include "mcrt_internal.h"
 
 using namespace mcrt;
@@ -66,6 +69,22 @@ void set_sun(DevScene& S, const float sun[3])
         S.sun[a] = sun[a];
         S.inv_sun[a] = sun[a] != 0.0f ? 1.0f / sun[a] : std::numeric_limits<float>::quiet_NaN();
     }
+}
+
+// Brings the pages of a caller's buffer in before the device writes them,
+// with their contents; where that cannot be (an older kernel, memory of another
+// kind) the copy does.  A copy to pages that nothing has touched yet faults
+// them in one by one from the device: means and standard errors of a 1024 x
+// 1024 image took up to 14 ms into new arrays, 0.2 into used ones; bringing
+// them in, beside the kernel before the copy, takes 0.5.
+void populate(void* p, size_t bytes)
+{
+#ifdef MADV_POPULATE_WRITE
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), a = reinterpret_cast<uintptr_t>(p), b = a & ~(page - 1);
+    if (bytes) (void)madvise(reinterpret_cast<void*>(b), (size_t)(a + bytes - b), MADV_POPULATE_WRITE);
+#else
+    (void)p; (void)bytes;
+#endif
 }
 
 bool finite_pos(float x) { return std::isfinite(x) && x > 0.0f; }
@@ -1721,6 +1740,8 @@ int mcrt_tally_read(const mcrt_tally* t, double* mean, double* se, uint64_t* n, 
         LAUNCH(ctx, launch_finalize(t->d_s1, t->d_s2, (double)t->n_per_cell, (int)m,
                                     t->cell_n.empty() ? nullptr : t->d_cell_n, t->nq, t->d_out, ctx->stream));
         cudaError_t e = cudaSuccess;
+        if (mean) populate(mean, m * sizeof(double));
+        if (se) populate(se, m * sizeof(double));
         if (mean) e = cudaMemcpyAsync(mean, t->d_out, m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
         if (se && e == cudaSuccess)
             e = cudaMemcpyAsync(se, t->d_out + m, m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
