@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256) oct_bricks_kernel(const void* __restrict_
 // bytes written per 2^3 voxels, 16 per lane.  For the 1024 x 1024 x 160 field:
 // one thread per cell walking down from the top level 162 us, one warp per
 // brick with a lane per level 104 us, this 52 us.  finest: 0 (voxel leaves)
-// to 2.
+// or 1.
 __global__ void __launch_bounds__(256) oct_leafmap_kernel(LevelTable T, int levels, int finest, float tau, int nbx,
                                                           int nby, unsigned nbricks, uint2* __restrict__ leaf)
 {
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(256) oct_leafmap_kernel(LevelTable T, int leve
         } else if (levels >= 2) {
             const size_t c = ((size_t)(cz >> 1) * T.dims[2][1] + (cy >> 1)) * T.dims[2][0] + (cx >> 1);
             const float M = T.p[2][c];
-            if (finest == 2 || __fmul_rn(M, T.hz[2]) <= tau) {
+            if (__fmul_rn(M, T.hz[2]) <= tau) {
                 e[0] = e[1] = entry(M, T.pmin[2][c], 2);
                 done = true;
             }
@@ -429,7 +429,6 @@ cudaError_t launch_leafmap(const mcrt_scene* sc, float tau, int finest, int grid
     }
     const long long cells = (long long)sc->nb[0] * sc->nb[1] * sc->nb[2];
     if (oct) {
-        if (finest > 2) return cudaErrorInvalidValue;
         oct_leafmap_kernel<<<(unsigned)((cells + 31) / 32), 256, 0, st>>>(T, levels, finest, tau, sc->nb[0], sc->nb[1],
                                                                         (unsigned)cells, sc->d_oleaf);
     } else {

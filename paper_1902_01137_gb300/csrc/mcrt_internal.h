@@ -196,8 +196,7 @@ struct TraceParams {
     int max_order;
     int sun_mode;
     uint32_t max_steps;
-    int rare_batch;            // lanes waiting for a rare phase that trigger it
-    int min_steppers;          // below this many stepping lanes, run rare phases anyway
+    int min_steppers;          // below this many stepping lanes, those that wait get their rare pass
     int claim_lanes;           // lanes of a warp that claim paths; the others only help
     // camera
     int width, height;
@@ -261,8 +260,8 @@ struct TraceParams {
 constexpr int kDefaultRareBatch = 16, kDefaultRareBatchLong = 20;
 inline void set_rare_batch(TraceParams& P, int requested, bool learned = false)
 {
-    P.rare_batch = requested > 0 ? requested : (P.S.hf || learned ? kDefaultRareBatchLong : kDefaultRareBatch);
-    P.min_steppers = 33 - P.rare_batch;
+    const int wait = requested > 0 ? requested : (P.S.hf || learned ? kDefaultRareBatchLong : kDefaultRareBatch);
+    P.min_steppers = 33 - wait;
 }
 
 inline void set_key(TraceParams& P, uint64_t seed)

@@ -61,7 +61,6 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 enum Kind { kMain = 0, kSunLocal = 1, kSunDirect = 2, kSunHelp = 3 };   // kSunHelp: another lane's kSunLocal
-enum Event { EV_NONE = 0, EV_REAL, EV_GROUND, EV_ESCAPE, EV_SUN_END, EV_ABORT };
 
 // Counter slots (see mcrt_tally_counters).
 enum {

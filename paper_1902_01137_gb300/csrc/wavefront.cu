@@ -121,13 +121,6 @@ __device__ __forceinline__ void wf_tally(const TraceParams& P, uint32_t cell, fl
     atomicAdd(P.s2 + cell, (double)(score * score));
 }
 
-// A ray from o along unit d: its voxel, leaf and exit distance.
-template <bool BF16>
-__device__ __forceinline__ void wf_ray_start(const DevScene& S, Ray& R, const float o[3], const float d[3])
-{
-    ray_begin<BF16>(S, R, o, d);
-}
-
 // A stage kernel's threads are persistent: a lane that finishes its entry
 // takes the next one from the queue, so a warp does not wait for its
 // slowest entry.  Idle lanes refill together, once kRefillLanes of them are
@@ -213,7 +206,7 @@ __global__ void __launch_bounds__(kWfBlock) wf_flight_kernel(const __grid_consta
             tau = F.aux[i];
             blk = F.blk[i];
             if (blk == 0u) {
-                wf_ray_start<BF16>(S, R, o, d);
+                ray_begin<BF16>(S, R, o, d);
                 blk = 1;
             } else {
                 // a flight suspended at its step budget: re-entering its
@@ -357,7 +350,7 @@ __global__ void __launch_bounds__(kWfBlock) wf_vertex_kernel(const __grid_consta
             if (trk) {
                 // the sun ray: T_sun by ratio (or delta) tracking
                 Ts = 1.0f;
-                wf_ray_start<BF16>(S, R, vx, S.sun);
+                ray_begin<BF16>(S, R, vx, S.sun);
                 tau = -__logf(u01(x.w));
                 blk = 1;
             }
