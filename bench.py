@@ -67,22 +67,22 @@ WORKLOAD = "cumulus 512x512x160 @25m, 3-level majorants, 1024x1024 nadir image x
 W, H, SPP = CUMULUS.image.width, CUMULUS.image.height, CUMULUS.image.spp
 # DRAM traffic of the trace kernel from the last full ncu capture (profiles/),
 # valid only while the kernel's sources are the ones that were captured
-PROFILED_TRACE_SHA = "aa804485da4a1be7"
-PROFILED_DRAM_BYTES_PER_PATH = 23.28
+PROFILED_TRACE_SHA = "702d8e17e31def95"
+PROFILED_DRAM_BYTES_PER_PATH = 23.38
 # issue figures: warp instructions per path and threads per warp instruction
 # from a one-pass count of a bench launch (1024^2 x 64 spp), the small
 # capture's issue-active fraction; the kernel is issue-bound, so these
 # locate it against its real ceiling: 152 SMs x 4 schedulers x 1 warp
 # instruction per cycle
-PROFILED_ISSUE_ACTIVE = 0.7665
+PROFILED_ISSUE_ACTIVE = 0.768
 PROFILED_THREADS_PER_INST = 15.63
-PROFILED_WARP_INST_PER_PATH = 2853.5
+PROFILED_WARP_INST_PER_PATH = 2846.6
 PROFILED_SOURCE = "profiles/trace_kernel_cumulus_1024px64spp_launches.md"
 # the same capture over the octree (profiles/trace_kernel_octree_cumulus_512px16spp_ncu_full.md)
-PROFILED_OCTREE_DRAM_BYTES_PER_PATH = 38.59
+PROFILED_OCTREE_DRAM_BYTES_PER_PATH = 38.50
 # one-pass count of the bench's octree launches (same profile as the pyramid's)
-PROFILED_OCTREE_WARP_INST_PER_PATH = 2601.4
-PROFILED_OCTREE_THREADS_PER_INST = 14.52
+PROFILED_OCTREE_WARP_INST_PER_PATH = 2596.4
+PROFILED_OCTREE_THREADS_PER_INST = 14.51
 
 
 def trace_sources_sha() -> str:

@@ -85,10 +85,12 @@ enum { MCRT_GRID_PYRAMID = 0, MCRT_GRID_OCTREE = 1 };
 enum { MCRT_ORDER_COST = 0, MCRT_ORDER_RASTER = 1 };
 
 /* How a camera trace schedules its paths on the GPU (mcrt_trace_opts.schedule).
- * PERSISTENT: one loop per GPU thread that takes one step of one path per
- * iteration, path state in registers (the default).  WAVEFRONT: paths wait
- * in structure-of-arrays queues in device memory between stages (flight
- * tracking; vertex and sun ray; path start), one kernel per stage and round.
+ * PERSISTENT: every GPU thread carries one path at a time, in a kernel that
+ * alternates between traversal steps and passes over everything rarer, the
+ * traversal's state in registers and the rest in shared memory (the default).
+ * WAVEFRONT: paths wait in structure-of-arrays queues in device memory between
+ * stages (flight tracking; vertex and sun ray; path start), one kernel per
+ * stage and round.
  * Both compute the same path scores bit for bit (Philox counters and FP32
  * steps are the same); only the order of the FP64 tally additions differs.
  * The wavefront form serves plain camera images only: no proposal, shards,
@@ -229,7 +231,8 @@ MCRT_API int mcrt_scene_set_clear_sky_phase(mcrt_scene* scene, int32_t phase);
  * FP32 heights [km] (x fastest) at the corners of a periodic grid of
  * hnx x hny cells spanning the field's x-y extent; each cell is cut along
  * the diagonal from corner (i, j) to (i+1, j+1) into two planar triangles.
- * mem: MCRT_MEM_HOST or MCRT_MEM_DEVICE (borrowed for the call, copied).
+ * mem: MCRT_MEM_HOST or MCRT_MEM_DEVICE (borrowed for the call, copied; the
+ * scene holds 16 bytes a cell, beyond 2^28 cells 4, and the max pyramid).
  * Heights must be finite and in [0, nz * dz] (MCRT_ERR_ARG otherwise).
  * Paths end their flights on the surface, sun rays that meet it are
  * shadowed, ground vertices use the facet normal (Lambertian about it,

@@ -34,8 +34,9 @@
 // first optical depth), a Rayleigh vertex its species from word 0 of block
 // kBlockVertex.
 //
-// What bounds it: instruction issue.  The split keeps the step loop short
-// (no random block, sums, claims or path state in it) and its registers few
+// What bounds it: instruction issue.  The split keeps the step loop short (no
+// sums, claims or path state in it, and of the random blocks only that of a
+// tentative collision in a leaf of several voxels) and its registers few
 // enough for 8 blocks of 128 threads an SM without spills; a single loop
 // with everything in it, at 72 registers and one Philox block per iteration,
 // took 95.1 ms for 16.8 M paths of the 512 x 512 x 160 cumulus image, this
